@@ -76,6 +76,51 @@ sk_status dalloc(T** p, size_t bytes) {
     return SK_OK;
 }
 
+// Stream-ordered workspace of calls that need some only while they run, from
+// one memory pool per device: up to kWorkspaceKept bytes stay with the pool
+// between calls (a cudaMalloc / cudaFree pair of the 80 MB an energy call at
+// N = 2048 takes costs more than its kernels), more goes back at the next
+// synchronisation, and all of it when the process's last instance is
+// destroyed.  The runtime's pools are safe for concurrent threads and order
+// reuse between streams.
+constexpr uint64_t kWorkspaceKept = 256ull << 20;
+std::mutex g_pool_mu;
+cudaMemPool_t g_pools[64] = {};
+std::atomic<int> g_instances{0};
+
+cudaMemPool_t workspace_pool() {
+    int dev = 0;
+    if (cudaGetDevice(&dev) != cudaSuccess || dev < 0 || dev >= 64) return nullptr;
+    std::lock_guard<std::mutex> lock(g_pool_mu);
+    if (!g_pools[dev]) {
+        cudaMemPoolProps p{};
+        p.allocType = cudaMemAllocationTypePinned;
+        p.location.type = cudaMemLocationTypeDevice;
+        p.location.id = dev;
+        uint64_t keep = kWorkspaceKept;
+        if (cudaMemPoolCreate(&g_pools[dev], &p) != cudaSuccess ||
+            cudaMemPoolSetAttribute(g_pools[dev], cudaMemPoolAttrReleaseThreshold, &keep) != cudaSuccess) {
+            cudaGetLastError();
+            g_pools[dev] = nullptr;
+        }
+    }
+    return g_pools[dev];
+}
+void workspace_trim() {
+    std::lock_guard<std::mutex> lock(g_pool_mu);
+    for (cudaMemPool_t p : g_pools)
+        if (p) cudaMemPoolTrimTo(p, 0);
+}
+sk_status ws_alloc(void** p, size_t bytes, cudaStream_t st) {
+    *p = nullptr;
+    cudaMemPool_t pool = workspace_pool();
+    const cudaError_t e = pool ? cudaMallocFromPoolAsync(p, bytes, pool, st) : cudaErrorMemoryAllocation;
+    if (e == cudaSuccess) return SK_OK;
+    cudaGetLastError();
+    *p = nullptr;
+    return fail(SK_ERR_OOM, "workspace of %zu bytes: %s", bytes, cudaGetErrorString(e));
+}
+
 // +-J weight tables (exact integer arithmetic on both the chain and its
 // checks): MCMCMC W[d] = round(2^52 exp(-2 beta_eff d)) for d = (dE - min)/2
 // until the first entry that rounds to zero; Metropolis M[k] =
@@ -619,6 +664,7 @@ sk_status sk_create_instance(uint32_t N, uint32_t kind, const void* couplings, u
         delete in;
         return s;
     }
+    g_instances++;
     *out = in;
     return SK_OK;
 }
@@ -679,6 +725,7 @@ sk_status sk_destroy_instance(sk_instance* in) {
     cudaEventDestroy(in->ev_main);
     cudaStreamDestroy(in->side);
     delete in;
+    if (--g_instances == 0) workspace_trim();
     return SK_OK;
 }
 
@@ -686,36 +733,63 @@ sk_status sk_energy(const sk_instance* in, const int8_t* spins, uint32_t count, 
                     double* out_E) {
     if (!in || !spins || !out_E) return fail(SK_ERR_INVALID_ARG, "NULL argument");
     if (count == 0) return SK_OK;
-    const size_t n = static_cast<size_t>(count) * in->N;
-    int8_t* tmp = nullptr;
-    double* dE = nullptr;
-    const int8_t* dsp = spins;
-    sk_status s = SK_OK;
-    if (mem == SK_MEM_HOST) {
-        for (size_t i = 0; i < n; ++i)
-            if (spins[i] != 1 && spins[i] != -1) return fail(SK_ERR_INVALID_ARG, "spin %zu is not +-1", i);
-        if ((s = dalloc(&tmp, n)) != SK_OK) return s;
-        const cudaError_t e = cudaMemcpyAsync(tmp, spins, n, cudaMemcpyHostToDevice, in->st);
-        if (e != cudaSuccess) {
-            cudaFree(tmp);
-            return fail(SK_ERR_CUDA, "sk_energy: %s", cudaGetErrorString(e));
-        }
-        dsp = tmp;
-    } else if (mem != SK_MEM_DEVICE) {
+    if (mem != SK_MEM_HOST && mem != SK_MEM_DEVICE)
         return fail(SK_ERR_INVALID_ARG, "mem must be SK_MEM_HOST or SK_MEM_DEVICE");
-    }
+    const size_t n = static_cast<size_t>(count) * in->N;
+    const bool host = mem == SK_MEM_HOST;
+    // host spins are checked before anything is written: here when they are
+    // few (two launches and a copy back cost ~10 us), else on the device
+    const bool check_here = host && n <= 16384;
+    for (size_t i = 0; check_here && i < n; ++i)
+        if (spins[i] != 1 && spins[i] != -1) return fail(SK_ERR_INVALID_ARG, "spin %zu is not +-1", i);
+    auto up = [](size_t b) { return (b + 1023u) & ~static_cast<size_t>(1023u); };
+    // workspace: the result of the spins' check, the energies, the column
+    // parts of the direct sum, host spins, the tensor path's operands
     const size_t tiles = sk::energy_tiles(in->N, count);
-    if ((s = dalloc(&dE, count * (1 + tiles) * sizeof(double))) != SK_OK) {
-        cudaFree(tmp);
-        return s;
+    const size_t o_E = 1024, o_part = o_E + up(count * sizeof(double));
+    const size_t o_spins = o_part + up(tiles > 1 ? tiles * count * sizeof(double) : 0);
+    const size_t o_tc = o_spins + (host ? up(n) : 0);
+    bool tc = sk::energy_on_tensor(in->kind, in->N, count);
+    void* ws = nullptr;
+    sk_status s = SK_ERR_OOM;
+    if (tc) s = ws_alloc(&ws, o_tc + sk::energy_workspace(in->kind, in->Npad, count), in->st);
+    if (s != SK_OK) {  // no room for the operands: the direct sum
+        tc = false;
+        if ((s = ws_alloc(&ws, o_tc, in->st)) != SK_OK) return s;
     }
-    cudaError_t e = sk::launch_energy(in->dJ, in->kind, in->N, in->Npad, in->scale, dsp, count, dE, in->st,
-                                      tiles > 1 ? dE + count : nullptr);
-    if (e == cudaSuccess) e = cudaMemcpyAsync(out_E, dE, count * sizeof(double), cudaMemcpyDeviceToHost, in->st);
-    if (e == cudaSuccess) e = cudaStreamSynchronize(in->st);
-    cudaFree(tmp);
-    cudaFree(dE);
+    unsigned char* base = static_cast<unsigned char*>(ws);
+    unsigned long long* dflag = reinterpret_cast<unsigned long long*>(base);
+    double* dE = reinterpret_cast<double*>(base + o_E);
+    const int8_t* dsp = spins;
+    std::vector<double> hE(count);
+    unsigned long long hflag = ~0ull;
+    int herr = 0;
+    cudaError_t e = cudaSuccess;
+    if (host) {
+        dsp = reinterpret_cast<const int8_t*>(base + o_spins);
+        e = cudaMemcpyAsync(base + o_spins, spins, n, cudaMemcpyHostToDevice, in->st);
+    }
+    if (host && !check_here) {
+        if (e == cudaSuccess) e = sk::launch_check_spins(dsp, n, dflag, in->st);
+        if (e == cudaSuccess) e = cudaMemcpyAsync(&hflag, dflag, sizeof hflag, cudaMemcpyDeviceToHost, in->st);
+    }
+    const uint32_t* slices = nullptr;
+    const int* err = nullptr;
+    if (e == cudaSuccess && tc)
+        e = sk::launch_energy_tensor(in->dJ, in->kind, in->N, in->Npad, in->scale, dsp, count, dE, base + o_tc, &slices,
+                                     &err, in->st);
+    if (e == cudaSuccess && !(tc && in->kind == SK_J_PM1))  // (Gaussian: writes only if the launch above did not)
+        e = sk::launch_energy(in->dJ, in->kind, in->N, in->Npad, in->scale, dsp, count, dE, in->st,
+                              tiles > 1 ? reinterpret_cast<double*>(base + o_part) : nullptr, slices);
+    if (e == cudaSuccess) e = cudaMemcpyAsync(hE.data(), dE, count * sizeof(double), cudaMemcpyDeviceToHost, in->st);
+    if (e == cudaSuccess && err) e = cudaMemcpyAsync(&herr, err, sizeof herr, cudaMemcpyDeviceToHost, in->st);
+    cudaFreeAsync(ws, in->st);
+    const cudaError_t e2 = cudaStreamSynchronize(in->st);
+    if (e == cudaSuccess) e = e2;
     if (e != cudaSuccess) return fail(SK_ERR_CUDA, "sk_energy: %s", cudaGetErrorString(e));
+    if (hflag != ~0ull) return fail(SK_ERR_INVALID_ARG, "spin %llu is not +-1", hflag >> 2);
+    if (herr) return fail(SK_ERR_TIMEOUT, "sk_energy: a bounded device wait expired");
+    std::memcpy(out_E, hE.data(), count * sizeof(double));
     return SK_OK;
 }
 

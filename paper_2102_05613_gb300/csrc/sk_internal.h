@@ -139,9 +139,18 @@ cudaError_t launch_check_spins(const int8_t* s, uint64_t n, unsigned long long* 
 // columns of J are split over several CTAs per block of configurations;
 // without it one CTA covers all columns.
 uint32_t energy_tiles(uint32_t N, uint32_t count);
+// unless: a device word; when given and not 0 the launch writes nothing.
 cudaError_t launch_energy(const void* J, uint32_t kind, uint32_t N, uint32_t Npad, double scale,
                           const int8_t* spins, uint32_t count, double* out, cudaStream_t st,
-                          double* partial = nullptr);
+                          double* partial = nullptr, const uint32_t* unless = nullptr);
+// The same energies as exact products on the tensor cores (sk_recompute.cu).
+// The kernels leave 0 in *slices_word where they do not apply (Gaussian
+// couplings that span more than 62 bits) and write nothing then.
+bool energy_on_tensor(uint32_t kind, uint32_t N, uint32_t count);
+size_t energy_workspace(uint32_t kind, uint32_t npad, uint32_t count);
+cudaError_t launch_energy_tensor(const void* J, uint32_t kind, uint32_t N, uint32_t npad, double scale,
+                                 const int8_t* spins, uint32_t count, double* out, void* ws,
+                                 const uint32_t** slices_word, const int** err_word, cudaStream_t st);
 
 // Cluster-per-chain layout (sk_cluster*.cu): a cluster of C CTAs (1, 2, 4,
 // 8 or 16) holds W chains of one run (one warp per chain in each CTA; W = 1,

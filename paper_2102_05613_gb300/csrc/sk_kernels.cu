@@ -394,7 +394,9 @@ template <typename JT>
 __global__ void __launch_bounds__(256) energy_kernel(const JT* __restrict__ J, uint32_t N, uint32_t npad,
                                                       double scale, const int8_t* __restrict__ spins,
                                                       uint32_t count, double* __restrict__ out,
-                                                      double* __restrict__ partial) {
+                                                      double* __restrict__ partial,
+                                                      const uint32_t* __restrict__ unless) {
+    if (unless && *unless) return;  // the tensor-core launch before this one wrote the energies
     using A = typename std::conditional<sizeof(JT) == 1, int, double>::type;
     constexpr uint32_t CB = kEnergyChains;
     extern __shared__ __align__(16) unsigned char sb[];
@@ -449,7 +451,8 @@ __global__ void __launch_bounds__(256) energy_kernel(const JT* __restrict__ J, u
 }
 
 __global__ void energy_finish(const double* __restrict__ partial, uint32_t tiles, uint32_t count, double scale,
-                              double* __restrict__ out) {
+                              double* __restrict__ out, const uint32_t* __restrict__ unless) {
+    if (unless && *unless) return;
     const uint32_t c = blockIdx.x * blockDim.x + threadIdx.x;
     if (c >= count) return;
     double v = 0.0;
@@ -607,17 +610,18 @@ uint32_t energy_tiles(uint32_t N, uint32_t count) {
 }
 
 cudaError_t launch_energy(const void* J, uint32_t kind, uint32_t N, uint32_t Npad, double scale,
-                          const int8_t* spins, uint32_t count, double* out, cudaStream_t st, double* partial) {
+                          const int8_t* spins, uint32_t count, double* out, cudaStream_t st, double* partial,
+                          const uint32_t* unless) {
     const size_t sm = (N + 15) / 16 * 16;
     const uint32_t tiles = partial ? energy_tiles(N, count) : 1u;
     const dim3 grid((count + kEnergyChains - 1) / kEnergyChains, tiles);
     if (kind == 0)
         energy_kernel<int8_t><<<grid, 256, sm, st>>>(static_cast<const int8_t*>(J), N, Npad, scale, spins, count,
-                                                     out, partial);
+                                                     out, partial, unless);
     else
         energy_kernel<float><<<grid, 256, sm, st>>>(static_cast<const float*>(J), N, Npad, scale, spins, count,
-                                                    out, partial);
-    if (tiles > 1) energy_finish<<<(count + 255) / 256, 256, 0, st>>>(partial, tiles, count, scale, out);
+                                                    out, partial, unless);
+    if (tiles > 1) energy_finish<<<(count + 255) / 256, 256, 0, st>>>(partial, tiles, count, scale, out, unless);
     return cudaGetLastError();
 }
 

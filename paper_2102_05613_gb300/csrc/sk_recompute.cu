@@ -138,6 +138,12 @@ struct Args {
     uint32_t pm1;
     uint32_t fault;                 // kFaultWithholdTile: tests of the bounded waits
     uint32_t compute_only;          // tensor-pipe probe: operands loaded once, MMAs only
+    // energies (KIND 2): digit slices of J (device word, 0: none), and per
+    // slice and configuration the sum over n of s_n H_n
+    const uint32_t* nslices;
+    unsigned long long* esum;
+    uint32_t esum_stride;           // configurations in all (chains: those of this launch)
+    uint32_t b_row0, b_rows;        // the rows of J whose slices B holds
 };
 
 // Several operand sets in one launch: the tensor maps and arguments of each
@@ -298,16 +304,53 @@ __device__ __forceinline__ void epilogue_rows(uint32_t taddr, const Args& args, 
     __syncwarp();
 }
 
-// The persistent kernel.  BATCH: task t is tasks[t] of operand set
-// jobs[tasks[t].job] (maps in global memory, acquired before use); else the
-// maps and arguments are the kernel's parameters and task t is output tile
-// (t / tiles_n, t % tiles_n).
-template <bool F8, bool BATCH>
+// The energy epilogue for one warp: each lane adds s_n H_n of its row over the
+// warp's columns in int32 (H is an integer of at most 2^20: 128 columns stay
+// below 2^27) and adds the sum to the row's 64-bit word, exact in any order.
+__device__ __forceinline__ void energy_rows(uint32_t taddr, const Args& args, uint32_t row0, uint32_t n0, uint32_t c0,
+                                            uint32_t slice, bool tile_ok) {
+    const uint32_t row = row0 + (threadIdx.x & 31);
+    const bool row_ok = tile_ok && row < args.chains;
+    int isum = 0;
+#pragma unroll
+    for (uint32_t cb = 0; cb < NCB; ++cb) {
+        const uint32_t n = n0 + c0 + 32u * cb;
+        const bool ok = row_ok && n < args.npad;
+        uint4 sp[2];
+        if (ok) {
+            const uint4* p = reinterpret_cast<const uint4*>(args.s + static_cast<size_t>(row) * args.npad + n);
+            sp[0] = __ldg(p);
+            sp[1] = __ldg(p + 1);
+        }
+        uint32_t v[32];
+        tmem_ld32(taddr + c0 + 32u * cb, v);  // every lane: the load is warp-collective
+        if (!ok) continue;
+#pragma unroll
+        for (int k = 0; k < 32; ++k)
+            isum += sbyte32(word_of(sp[k >> 4], (k >> 2) & 3), k & 3) * __float2int_rn(__uint_as_float(v[k]));
+    }
+    if (row_ok && isum)
+        atomicAdd(&args.esum[static_cast<size_t>(slice) * args.esum_stride + row],
+                  static_cast<unsigned long long>(static_cast<long long>(isum)));
+    __syncwarp();
+}
+
+// The persistent kernel.  KIND 1 (a batch): task t is tasks[t] of operand set
+// jobs[tasks[t].job] (maps in global memory, acquired before use).  KIND 0:
+// the maps and arguments are the kernel's parameters and task t is output
+// tile (t / tiles_n, t % tiles_n).  KIND 2 (energies): B holds the digit
+// slices of the strict upper triangle of J one below the other; a task is one
+// slice of one output tile, whose K range starts at the tile's own columns
+// (what lies before them is zero), and the tasks with the longest range come
+// first, so that the last round of the persistent CTAs is a short one.
+template <bool F8, int KIND>
 __global__ void __launch_bounds__(WS_THREADS, 1)
     recompute_ws_kernel(const __grid_constant__ CUtensorMap tA, const __grid_constant__ CUtensorMap tB0,
                         const __grid_constant__ CUtensorMap tB1, const __grid_constant__ CUtensorMap tB2,
                         const Args args0, const BatchJob* __restrict__ jobs, const BatchTask* __restrict__ tasks,
                         uint32_t ntasks, uint32_t tiles_n) {
+    constexpr bool BATCH = KIND == 1;
+    constexpr bool ENERGY = KIND == 2;
     extern __shared__ __align__(1024) unsigned char smem_raw[];
     __shared__ __align__(8) uint64_t full[NS], empty[NS], tfull[2], tempty[2], drain;
     __shared__ uint32_t tmem_holder;
@@ -343,6 +386,11 @@ __global__ void __launch_bounds__(WS_THREADS, 1)
     asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
     const uint32_t tmem = tmem_holder;
 
+    const uint32_t tiles_m = ENERGY ? (args0.chains + BM - 1) / BM : 0u;
+    const uint32_t slices = ENERGY ? *args0.nslices : 0u;
+    if constexpr (ENERGY) ntasks = slices * tiles_m * tiles_n;
+    // energies: the slice of task t
+    auto slice_of = [&](uint32_t t) -> uint32_t { return ENERGY ? (t / tiles_m) % slices : 0u; };
     // the task's maps, arguments and tile origin
     auto task = [&](uint32_t t, const CUtensorMap*& A, const CUtensorMap* (&B)[3], const Args*& a, uint32_t& m0,
                     uint32_t& n0) {
@@ -362,8 +410,13 @@ __global__ void __launch_bounds__(WS_THREADS, 1)
             B[1] = &tB1;
             B[2] = &tB2;
             a = &args0;
-            m0 = (t / tiles_n) * BM;
-            n0 = (t % tiles_n) * BN;
+            if constexpr (ENERGY) {
+                m0 = (t % tiles_m) * BM;
+                n0 = a->b_row0 + (t / (tiles_m * slices)) * BN;
+            } else {
+                m0 = (t / tiles_n) * BM;
+                n0 = (t % tiles_n) * BN;
+            }
         }
     };
 
@@ -382,7 +435,9 @@ __global__ void __launch_bounds__(WS_THREADS, 1)
                     for (int q = 0; q < 3; ++q)
                         asm volatile("fence.proxy.tensormap::generic.acquire.gpu [%0], 128;" ::"l"(B[q]) : "memory");
                 }
-                const uint32_t total = a->terms * a->kblocks;
+                const uint32_t kb0 = ENERGY ? n0 / kElems : 0u;  // (n0: a multiple of BN)
+                const uint32_t total = ENERGY ? a->kblocks - kb0 : a->terms * a->kblocks;
+                const uint32_t brow = ENERGY ? slice_of(t) * a->b_rows + n0 - a->b_row0 : n0;
                 for (uint32_t i = 0; i < total; ++i, ++g) {
                     const uint32_t st = g % NS;
                     if (a->compute_only && g >= NS) break;  // the probe fills the ring once
@@ -395,13 +450,13 @@ __global__ void __launch_bounds__(WS_THREADS, 1)
                         withheld = g;
                         continue;
                     }
-                    const uint32_t term = i / a->kblocks, kb = i % a->kblocks;
+                    const uint32_t term = ENERGY ? 0u : i / a->kblocks, kb = ENERGY ? kb0 + i : i % a->kblocks;
                     unsigned char* sa = smem + st * STAGE_BYTES;
                     asm volatile("mbarrier.arrive.expect_tx.shared::cta.b64 _, [%0], %1;" ::"r"(saddr(&full[st])),
                                  "r"(STAGE_BYTES)
                                  : "memory");
                     tma_2d(saddr(sa), A, static_cast<int>(kb * kElems), static_cast<int>(m0), saddr(&full[st]));
-                    tma_2d(saddr(sa + TILE_A), B[term], static_cast<int>(kb * kElems), static_cast<int>(n0),
+                    tma_2d(saddr(sa + TILE_A), B[term], static_cast<int>(kb * kElems), static_cast<int>(brow),
                            saddr(&full[st]));
                 }
             }
@@ -428,7 +483,7 @@ __global__ void __launch_bounds__(WS_THREADS, 1)
                 }
                 asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
                 const uint32_t acc = tmem + 256u * b;
-                const uint32_t total = a->terms * a->kblocks;
+                const uint32_t total = ENERGY ? a->kblocks - n0 / kElems : a->terms * a->kblocks;
                 for (uint32_t i = 0; i < total; ++i, ++g) {
                     const uint32_t st = g % NS;
                     // (the probe waits for each stage once, then reuses it)
@@ -450,8 +505,10 @@ __global__ void __launch_bounds__(WS_THREADS, 1)
             // every MMA issued has finished before the accumulators' tensor
             // memory is released (at once after a normal run; bounded after an
             // expired wait)
-            mma_commit(saddr(&drain));
-            wait_bounded(saddr(&drain), 0u);
+            if (j) {
+                mma_commit(saddr(&drain));
+                wait_bounded(saddr(&drain), 0u);
+            }
         }
     } else {
         // epilogue warps 2..9: tensor-memory lane quadrant warp % 4, column
@@ -468,7 +525,7 @@ __global__ void __launch_bounds__(WS_THREADS, 1)
             // the first column block's fields and spins do not depend on the
             // accumulator: their loads go out before the wait for it
             RowBlock first;
-            if (!a->compute_only)
+            if (!ENERGY && !a->compute_only)
                 load_row_block(first, *a, m0 + qd * 32u + lane, n0 + half * (BN / 2), m0 + qd * 32u + lane < a->chains);
             // every lane waits; the outcome is made warp-uniform
             const bool ok = __all_sync(0xffffffffu, !*vdead && wait_bounded(saddr(&tfull[b]), (j >> 1) & 1u));
@@ -478,7 +535,10 @@ __global__ void __launch_bounds__(WS_THREADS, 1)
             }
             asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
             const bool live = __all_sync(0xffffffffu, !*vdead);
-            if (!a->compute_only)
+            if constexpr (ENERGY)
+                energy_rows(tmem + ((qd * 32u) << 16) + 256u * b, *a, m0 + qd * 32u, n0, half * (BN / 2),
+                            slice_of(t), ok && live);
+            else if (!a->compute_only)
                 epilogue_rows(tmem + ((qd * 32u) << 16) + 256u * b, *a, m0 + qd * 32u, n0, half * (BN / 2),
                               ok && live, first);
             asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
@@ -745,16 +805,16 @@ cudaError_t launch_set_fields_batch(uint32_t kind, const RecomputeSet* sets, uin
         const uint32_t nt = static_cast<uint32_t>(tasks.size());
         const uint32_t grid = std::max<uint32_t>(1u, std::min<uint32_t>(nt, static_cast<uint32_t>(sm_count())));
         if (bf) {
-            e = cudaFuncSetAttribute(recompute_ws_kernel<false, true>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+            e = cudaFuncSetAttribute(recompute_ws_kernel<false, 1>, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                      SMEM_BYTES);
             if (e == cudaSuccess)
-                recompute_ws_kernel<false, true><<<grid, WS_THREADS, SMEM_BYTES, st>>>(none, none, none, none, a0,
+                recompute_ws_kernel<false, 1><<<grid, WS_THREADS, SMEM_BYTES, st>>>(none, none, none, none, a0,
                                                                                       djobs, dtasks, nt, 0u);
         } else {
-            e = cudaFuncSetAttribute(recompute_ws_kernel<true, true>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+            e = cudaFuncSetAttribute(recompute_ws_kernel<true, 1>, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                      SMEM_BYTES);
             if (e == cudaSuccess)
-                recompute_ws_kernel<true, true><<<grid, WS_THREADS, SMEM_BYTES, st>>>(none, none, none, none, a0,
+                recompute_ws_kernel<true, 1><<<grid, WS_THREADS, SMEM_BYTES, st>>>(none, none, none, none, a0,
                                                                                      djobs, dtasks, nt, 0u);
         }
         if (e == cudaSuccess) e = cudaGetLastError();
@@ -837,7 +897,7 @@ cudaError_t launch_recompute(uint32_t kind, const int8_t* s, void* h, float* out
     // between the conversion and the main kernel stays short
     CUtensorMap tA, tB[3];
     if ((e = cached_maps(s_op, j_op, bf, chains, npad, &tA, tB)) != cudaSuccess) return e;
-    Args a;
+    Args a{};
     a.h = h;
     a.s = s;
     a.out = out;
@@ -859,17 +919,290 @@ cudaError_t launch_recompute(uint32_t kind, const int8_t* s, void* h, float* out
     if (nt == 0) return cudaSuccess;
     const uint32_t grid = std::min<uint32_t>(nt, static_cast<uint32_t>(sm_count()));
     if (bf) {
-        if ((e = smem_attribute(recompute_ws_kernel<false, false>, 0)) != cudaSuccess) return e;
-        recompute_ws_kernel<false, false><<<grid, WS_THREADS, SMEM_BYTES, st>>>(tA, tB[0], tB[1], tB[2], a, nullptr,
+        if ((e = smem_attribute(recompute_ws_kernel<false, 0>, 0)) != cudaSuccess) return e;
+        recompute_ws_kernel<false, 0><<<grid, WS_THREADS, SMEM_BYTES, st>>>(tA, tB[0], tB[1], tB[2], a, nullptr,
                                                                                nullptr, nt, tiles_n);
     } else {
-        if ((e = smem_attribute(recompute_ws_kernel<true, false>, 1)) != cudaSuccess) return e;
-        recompute_ws_kernel<true, false><<<grid, WS_THREADS, SMEM_BYTES, st>>>(tA, tB[0], tB[0], tB[0], a, nullptr,
+        if ((e = smem_attribute(recompute_ws_kernel<true, 0>, 1)) != cudaSuccess) return e;
+        recompute_ws_kernel<true, 0><<<grid, WS_THREADS, SMEM_BYTES, st>>>(tA, tB[0], tB[0], tB[0], a, nullptr,
                                                                               nullptr, nt, tiles_n);
     }
     e = cudaGetLastError();
     if (e != cudaSuccess || mode >= 2 || a.cnt) return e;
     finish_energy<<<(chains + 255) / 256, 256, 0, st>>>(dE, chains, scale, stats);
+    return cudaGetLastError();
+}
+
+// ---------------------------------------------------------------------------
+// Energies of many configurations (sk_energy) as products on the tensor cores
+// ---------------------------------------------------------------------------
+// E(c) = -scale sum_n s_n H_n, H_n = sum_{k > n} J_nk s_k: a product with the
+// strict upper triangle of J, taken exactly.  +-J: one FP8 slice.  Gaussian:
+// every J_ij is an integer q_ij times 2^lsb, lsb the lowest bit set in any of
+// them; q is written as signed base-256 digits, each exact in bf16, and a
+// digit's sums stay below 2^20 (128 x 8192), exact in the FP32 accumulator.
+// The digits' energy sums are integers (int32 per tile row, int64 per
+// configuration) joined in 128 bits, so the result is rounded once, where the
+// double-precision sum it replaces (energy_kernel) rounds at every term: the
+// error against a 64-bit product is the same 1.1e-16 (N = 2048).  Couplings
+// that span more than kEnergyBits bits take energy_kernel.  Bound: FP64 adds
+// run at 2 per clock and SM on this part; the 7 slices a Gaussian matrix of
+// N = 2048 needs are 3e10 bf16 multiply-adds for 2048 configurations (half
+// the matrix): 12.35 ms a call -> 0.14 ms, of which the fixed cost is 0.07.
+namespace {
+constexpr uint32_t kEnergyBits = 62;  // q fits a signed 64-bit integer and 8 digits
+constexpr uint32_t kEnergySlices = 8;
+
+// Header of the workspace: [0] slices (0: take energy_kernel), [1] lowest bit
+// set in any coupling, [2] highest (biased by 256, running min / max), [3] error word.
+struct EnergyHead {
+    uint32_t slices;
+    uint32_t lsb, msb;
+    int err;
+};
+
+// The position of the lowest and highest set bits of |x|, biased by 256.
+__device__ __forceinline__ void bits_of(float x, uint32_t& lo, uint32_t& hi) {
+    const uint32_t b = __float_as_uint(x) & 0x7FFFFFFFu;
+    if (b == 0u) return;
+    const uint32_t e = b >> 23;
+    const uint32_t m = (b & 0x7FFFFFu) | (e ? 0x800000u : 0u);
+    const uint32_t base = (e ? e : 1u) + 256u - 150u;
+    lo = min(lo, base + static_cast<uint32_t>(__ffs(static_cast<int>(m)) - 1));
+    hi = max(hi, base + 31u - static_cast<uint32_t>(__clz(static_cast<int>(m))));
+}
+__global__ void energy_range(const float* __restrict__ J, uint64_t words4, EnergyHead* __restrict__ head) {
+    uint32_t lo = 0xFFFFFFFFu, hi = 0u;
+    for (uint64_t i = blockIdx.x * static_cast<uint64_t>(blockDim.x) + threadIdx.x; i < words4;
+         i += static_cast<uint64_t>(gridDim.x) * blockDim.x) {
+        const float4 v = __ldg(reinterpret_cast<const float4*>(J) + i);
+        bits_of(v.x, lo, hi);
+        bits_of(v.y, lo, hi);
+        bits_of(v.z, lo, hi);
+        bits_of(v.w, lo, hi);
+    }
+    lo = __reduce_min_sync(0xffffffffu, lo);
+    hi = __reduce_max_sync(0xffffffffu, hi);
+    if ((threadIdx.x & 31) == 0) {
+        atomicMin(&head->lsb, lo);
+        atomicMax(&head->msb, hi);
+    }
+}
+
+// Slices of rows row0 .. row0 + gridDim.x - 1 of the strict upper triangle,
+// slice t of row row0 + r at row t gridDim.x + r: the columns from the start
+// of the row's own tile on (the rest is not read).  A thread writes 8 columns
+// (16 bytes) of every slice.
+__global__ void energy_slices(const float* __restrict__ J, uint16_t* __restrict__ out, uint32_t npad, uint32_t row0,
+                              EnergyHead* __restrict__ head) {
+    const uint32_t lsb = head->lsb, msb = head->msb;
+    const uint32_t bits = msb >= lsb ? msb - lsb + 1u : 0u;  // none set: all couplings zero
+    const uint32_t S = bits > kEnergyBits ? 0u : (bits + 2u + 7u) / 8u;
+    if (blockIdx.x == 0 && threadIdx.x == 0) head->slices = S;
+    const uint32_t n = row0 + blockIdx.x;
+    for (uint32_t k = (n & ~(BN - 1u)) + 8u * threadIdx.x; S && k < npad; k += 8u * blockDim.x) {
+        float x[8];
+        *reinterpret_cast<float4*>(&x[0]) = __ldg(reinterpret_cast<const float4*>(J + static_cast<size_t>(n) * npad + k));
+        *reinterpret_cast<float4*>(&x[4]) = __ldg(reinterpret_cast<const float4*>(J + static_cast<size_t>(n) * npad + k + 4));
+        long long q[8];
+#pragma unroll
+        for (int e = 0; e < 8; ++e) {
+            const uint32_t b = __float_as_uint(x[e]), f = (b >> 23) & 255u;
+            const long long m = (b & 0x7FFFFFu) | (f ? 0x800000u : 0u);
+            const int sh = static_cast<int>((f ? f : 1u) + 256u - 150u) - static_cast<int>(lsb);
+            const long long a = m == 0 ? 0ll : sh >= 0 ? m << sh : m >> -sh;  // (the bits shifted out are zero)
+            q[e] = k + e > n ? ((b >> 31) ? -a : a) : 0ll;
+        }
+        for (uint32_t t = 0; t < S; ++t) {
+            uint32_t w[4];
+#pragma unroll
+            for (int e = 0; e < 4; ++e) {
+                uint32_t p = 0;
+#pragma unroll
+                for (int h = 0; h < 2; ++h) {
+                    const int d = static_cast<int>(static_cast<int8_t>(q[2 * e + h] & 0xFF));
+                    q[2 * e + h] = (q[2 * e + h] - d) >> 8;
+                    p |= (__float_as_uint(static_cast<float>(d)) >> 16) << (16 * h);  // |d| <= 128: exact in bf16
+                }
+                w[e] = p;
+            }
+            *reinterpret_cast<uint4*>(out + (static_cast<size_t>(t) * gridDim.x + blockIdx.x) * npad + k) =
+                make_uint4(w[0], w[1], w[2], w[3]);
+        }
+    }
+}
+// The same for +-J: one slice of e4m3 bytes, 16 columns per thread.
+__global__ void energy_slice_pm1(const int8_t* __restrict__ J, uint8_t* __restrict__ out, uint32_t npad,
+                                 uint32_t row0, EnergyHead* __restrict__ head) {
+    if (blockIdx.x == 0 && threadIdx.x == 0) head->slices = 1u;
+    const uint32_t n = row0 + blockIdx.x;
+    for (uint32_t k = (n & ~(BN - 1u)) + 16u * threadIdx.x; k < npad; k += 16u * blockDim.x) {
+        const uint4 v = __ldg(reinterpret_cast<const uint4*>(J + static_cast<size_t>(n) * npad + k));
+        uint32_t w[4] = {v.x, v.y, v.z, v.w};
+#pragma unroll
+        for (uint32_t e = 0; e < 4; ++e) {
+            const uint32_t k0 = k + 4u * e;  // bytes of columns k > n only
+            const uint32_t keep = n < k0 ? 0xFFFFFFFFu : n >= k0 + 3u ? 0u : 0xFFFFFFFFu << (8u * (n + 1u - k0));
+            w[e] = e4m3_of4(w[e] & keep);
+        }
+        *reinterpret_cast<uint4*>(out + static_cast<size_t>(blockIdx.x) * npad + k) = make_uint4(w[0], w[1], w[2], w[3]);
+    }
+}
+// Configurations (rows x N, any alignment) as padded int8 rows and as the MMA
+// operand; a value below 0 counts as -1, any other as +1, padding 0.
+__global__ void energy_spins(const int8_t* __restrict__ spins, uint32_t N, uint32_t npad, uint32_t rows, uint32_t bf,
+                             int8_t* __restrict__ s, void* __restrict__ op) {
+    const uint32_t words = npad / 16u;
+    for (uint32_t c = blockIdx.x; c < rows; c += gridDim.x)
+        for (uint32_t wd = threadIdx.x; wd < words; wd += blockDim.x) {
+            const int8_t* src = spins + static_cast<size_t>(c) * N + 16u * wd;
+            uint32_t w[4];
+#pragma unroll
+            for (uint32_t e = 0; e < 4; ++e) {
+                w[e] = 0u;
+#pragma unroll
+                for (uint32_t h = 0; h < 4; ++h)
+                    if (16u * wd + 4u * e + h < N) w[e] |= (__ldg(src + 4u * e + h) < 0 ? 0xFFu : 0x01u) << (8u * h);
+            }
+            const uint4 v = make_uint4(w[0], w[1], w[2], w[3]);
+            const size_t at = static_cast<size_t>(c) * words + wd;
+            reinterpret_cast<uint4*>(s)[at] = v;
+            dev::spins_to_op16(op, at, v, bf != 0u);
+        }
+}
+// The slices' sums joined: E = -scale 2^lsb sum_t 256^t esum_t, in 128 bits.
+__global__ void energy_join(const unsigned long long* __restrict__ esum, const EnergyHead* __restrict__ head,
+                            uint32_t rows, double scale, uint32_t pm1, double* __restrict__ out) {
+    const uint32_t c = blockIdx.x * blockDim.x + threadIdx.x;
+    const uint32_t S = head->slices;
+    if (c >= rows || S == 0u) return;
+    unsigned long long lo = 0, hi = 0;  // two's complement
+    for (uint32_t t = S; t-- > 0u;) {
+        hi = (hi << 8) | (lo >> 56);
+        lo <<= 8;
+        const unsigned long long v = esum[static_cast<size_t>(t) * rows + c];
+        lo += v;
+        hi += (lo < v ? 1ull : 0ull) + static_cast<unsigned long long>(static_cast<long long>(v) >> 63);
+    }
+    const bool neg = static_cast<long long>(hi) < 0;
+    if (neg) {
+        lo = ~lo + 1ull;
+        hi = ~hi + (lo == 0ull ? 1ull : 0ull);
+    }
+    double v = fma(static_cast<double>(hi), 0x1p64, static_cast<double>(lo));
+    if (neg) v = -v;
+    if (!pm1) v = ldexp(v, S > 0u && head->msb >= head->lsb ? static_cast<int>(head->lsb) - 256 : 0);
+    out[c] = -scale * v;
+}
+
+// Configurations and rows of J a launch takes: operands of at most 96 MB each,
+// whole tiles of 128 and 256.
+uint32_t energy_chunk(uint32_t npad, uint32_t count) {
+    return std::min(count, std::max<uint32_t>(128u, ((96u << 20) / (3u * npad)) & ~127u));
+}
+uint32_t energy_rows_of(uint32_t kind, uint32_t npad) {
+    const uint32_t row = npad * (kind == 0 ? 1u : 2u * kEnergySlices);
+    return std::min(npad, std::max<uint32_t>(256u, ((96u << 20) / row) & ~255u));
+}
+size_t energy_up(size_t b) { return (b + 1023u) & ~static_cast<size_t>(1023u); }
+}  // namespace
+
+// Where the tensor path is the faster one (us a call, direct sum / tensor, on
+// one configuration and on 4096): Gaussian N = 32 61 / 73 and 74 / 79, N = 64
+// 83 / 71 and 97 / 82, N = 512 440 / 73 and 1668 / 90; +-J N = 256 61 / 67 and
+// 74 / 74, N = 512 94 / 66 and 145 / 72, N = 2048 247 / 70 and 1761 / 84.  The
+// tensor path has a few more launches (the fixed ~65 us), the direct sum costs
+// at least a column's length of dependent adds.
+bool energy_on_tensor(uint32_t kind, uint32_t N, uint32_t count) {
+    const uint64_t terms = static_cast<uint64_t>(N) * N * count;
+    return kind == 0 ? N >= 320u || terms >= (1ull << 29) : N >= 48u || terms >= (1ull << 24);
+}
+
+size_t energy_workspace(uint32_t kind, uint32_t npad, uint32_t count) {
+    const size_t C = energy_chunk(npad, count), R = energy_rows_of(kind, npad);
+    const size_t S = kind == 0 ? 1 : kEnergySlices;
+    return 1024 + energy_up(R * npad * (kind == 0 ? 1 : 2 * S)) + energy_up(C * npad) +
+           energy_up(C * npad * (kind == 0 ? 1 : 2)) + energy_up(count * S * 8);
+}
+
+// Energies of `count` configurations into out[count] in `ws`
+// (energy_workspace bytes, 1 KB aligned).  *slices_word: where the kernels
+// leave the slice count, 0 when the couplings span too many bits and the
+// caller's energy_kernel launch is the one that writes out.
+cudaError_t launch_energy_tensor(const void* J, uint32_t kind, uint32_t N, uint32_t npad, double scale,
+                                 const int8_t* spins, uint32_t count, double* out, void* ws, const uint32_t** slices_word,
+                                 const int** err_word, cudaStream_t st) {
+    const bool bf = kind != 0;
+    const uint32_t C = energy_chunk(npad, count), R = energy_rows_of(kind, npad), S = bf ? kEnergySlices : 1u;
+    unsigned char* p = static_cast<unsigned char*>(ws);
+    EnergyHead* head = reinterpret_cast<EnergyHead*>(p);
+    p += 1024;
+    void* jop = p;
+    p += energy_up(static_cast<size_t>(R) * npad * (bf ? 2 * S : 1));
+    int8_t* s = reinterpret_cast<int8_t*>(p);
+    p += energy_up(static_cast<size_t>(C) * npad);
+    void* sop = p;
+    p += energy_up(static_cast<size_t>(C) * npad * (bf ? 2 : 1));
+    unsigned long long* esum = reinterpret_cast<unsigned long long*>(p);
+    *slices_word = &head->slices;
+    *err_word = &head->err;
+    cudaError_t e = cudaMemsetAsync(head, 0, sizeof(EnergyHead), st);
+    if (e == cudaSuccess) e = cudaMemsetAsync(&head->lsb, 0xFF, sizeof(uint32_t), st);
+    if (e == cudaSuccess) e = cudaMemsetAsync(esum, 0, static_cast<size_t>(count) * S * 8, st);
+    if (e == cudaSuccess)
+        e = bf ? smem_attribute(recompute_ws_kernel<false, 2>, 2) : smem_attribute(recompute_ws_kernel<true, 2>, 3);
+    if (e != cudaSuccess) return e;
+    if (bf) {
+        const uint64_t w4 = static_cast<uint64_t>(npad) * npad / 4u;
+        energy_range<<<static_cast<uint32_t>(std::min<uint64_t>((w4 + 1023u) / 1024u, 608u)), 256, 0, st>>>(
+            static_cast<const float*>(J), w4, head);
+    }
+    for (uint32_t r0 = 0; r0 < npad; r0 += R) {
+        const uint32_t rows_j = std::min(R, npad - r0);
+        const uint32_t threads = std::min<uint32_t>(256u, std::max<uint32_t>(32u, (npad / (bf ? 8u : 16u) + 31u) & ~31u));
+        if (bf)
+            energy_slices<<<rows_j, threads, 0, st>>>(static_cast<const float*>(J), static_cast<uint16_t*>(jop), npad, r0, head);
+        else
+            energy_slice_pm1<<<rows_j, threads, 0, st>>>(static_cast<const int8_t*>(J), static_cast<uint8_t*>(jop), npad, r0,
+                                                        head);
+        if ((e = cudaGetLastError()) != cudaSuccess) return e;
+        CUtensorMap tB;
+        if ((e = make_map(&tB, jop, bf, static_cast<uint64_t>(S) * rows_j, npad, BN)) != cudaSuccess) return e;
+        for (uint32_t c0 = 0; c0 < count; c0 += C) {
+            const uint32_t rows = std::min(C, count - c0);
+            if (r0 == 0 || C < count) {  // (one block of configurations keeps its operand)
+                const uint32_t sth = std::min<uint32_t>(128u, std::max<uint32_t>(32u, (npad / 16u + 31u) & ~31u));
+                energy_spins<<<std::min<uint32_t>(rows, 2432u), sth, 0, st>>>(spins + static_cast<size_t>(c0) * N, N, npad,
+                                                                             rows, bf ? 1u : 0u, s, sop);
+                if ((e = cudaGetLastError()) != cudaSuccess) return e;
+            }
+            CUtensorMap tA;
+            if ((e = make_map(&tA, sop, bf, rows, npad, BM)) != cudaSuccess) return e;
+            Args a{};
+            a.s = s;
+            a.err = &head->err;
+            a.chains = rows;
+            a.npad = npad;
+            a.kblocks = (npad + (bf ? 63u : 127u)) / (bf ? 64u : 128u);
+            a.terms = 1;
+            a.pm1 = bf ? 0u : 1u;
+            a.nslices = &head->slices;
+            a.esum = esum + c0;
+            a.esum_stride = count;
+            a.b_row0 = r0;
+            a.b_rows = rows_j;
+            const uint32_t tiles_n = (rows_j + BN - 1) / BN;
+            const uint32_t grid = std::min<uint32_t>(S * tiles_n * ((rows + BM - 1) / BM), static_cast<uint32_t>(sm_count()));
+            if (bf)
+                recompute_ws_kernel<false, 2><<<grid, WS_THREADS, SMEM_BYTES, st>>>(tA, tB, tB, tB, a, nullptr, nullptr,
+                                                                                   0u, tiles_n);
+            else
+                recompute_ws_kernel<true, 2><<<grid, WS_THREADS, SMEM_BYTES, st>>>(tA, tB, tB, tB, a, nullptr, nullptr,
+                                                                                  0u, tiles_n);
+            if ((e = cudaGetLastError()) != cudaSuccess) return e;
+        }
+    }
+    energy_join<<<(count + 255u) / 256u, 256, 0, st>>>(esum, head, count, scale, bf ? 0u : 1u, out);
     return cudaGetLastError();
 }
 
@@ -907,15 +1240,15 @@ cudaError_t tensor_peak_probe(uint32_t kind, uint32_t tiles, uint32_t reps, cuda
     auto launch = [&]() {
         // task t: rows (t / 1) * BM, columns 0; each CTA's first task is its own block of A
         if (bf)
-            recompute_ws_kernel<false, false><<<grid, WS_THREADS, SMEM_BYTES, st>>>(tA, tB, tB, tB, a, nullptr,
+            recompute_ws_kernel<false, 0><<<grid, WS_THREADS, SMEM_BYTES, st>>>(tA, tB, tB, tB, a, nullptr,
                                                                                    nullptr, nt, 1u);
         else
-            recompute_ws_kernel<true, false><<<grid, WS_THREADS, SMEM_BYTES, st>>>(tA, tB, tB, tB, a, nullptr,
+            recompute_ws_kernel<true, 0><<<grid, WS_THREADS, SMEM_BYTES, st>>>(tA, tB, tB, tB, a, nullptr,
                                                                                   nullptr, nt, 1u);
         return cudaGetLastError();
     };
     if (e == cudaSuccess)
-        e = bf ? smem_attribute(recompute_ws_kernel<false, false>, 0) : smem_attribute(recompute_ws_kernel<true, false>, 1);
+        e = bf ? smem_attribute(recompute_ws_kernel<false, 0>, 0) : smem_attribute(recompute_ws_kernel<true, 0>, 1);
     if (e == cudaSuccess) e = launch();  // warm-up
     if (e == cudaSuccess) e = cudaEventCreate(&e0);
     if (e == cudaSuccess) e = cudaEventCreate(&e1);

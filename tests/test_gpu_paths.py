@@ -27,7 +27,7 @@ def test_start_spin_check_finds_the_first_bad_spin(offset, chains, N):
     run = sk.Run(inst, chains=chains, K=4, seed=2)
     view = buf[offset:offset + n]
     head = min(n, (16 - view.data_ptr() % 16) % 16)
-    for at in sorted({0, max(0, head - 1), min(head, n - 1), n // 2, max(head, n - (n - head) % 16 - 1), n - 1}):
+    for at in sorted({0, max(0, head - 1), min(head, n - 1), n // 2, min(n - 1, max(head, n - (n - head) % 16 - 1)), n - 1}):
         for bad in (0, 2, -2, -128, 127):
             view.copy_(good)
             view[at] = bad
@@ -41,3 +41,78 @@ def test_start_spin_check_finds_the_first_bad_spin(offset, chains, N):
     run.reset(view)
     assert np.array_equal(run.state()[0].reshape(-1), good.numpy())
     run.close(); inst.close()
+
+
+def _exact_energy(J, s, scale):
+    # correctly rounded sum of the couplings' signed values
+    import math
+    i, j = np.triu_indices(J.shape[0], 1)
+    return -scale * math.fsum((J[i, j].astype(np.float64) * s[i] * s[j]).tolist())
+
+
+def _sym(upper):
+    upper = np.triu(upper, 1)
+    return np.ascontiguousarray((upper + upper.T).astype(np.float32))
+
+
+@pytest.mark.parametrize("N,count", [(2, 1), (33, 127), (96, 128), (256, 129), (257, 40), (300, 700)])
+def test_energies_are_exact_products(N, count):
+    # tile edges of 128 configurations and 256 columns; +-J exact, Gaussian
+    # rounded once (and once more by the scale)
+    torch = need_gpu()
+    S = inputs.initial_spins(count, N, 5)
+    some = sorted({0, count // 2, count - 1})
+    for J in (inputs.couplings_pm1(N, 6), inputs.couplings_gauss(N, 7)):
+        inst = sk.Instance(J, scale=0.75)
+        E = inst.energy(S)
+        odd = torch.zeros(count * N + 3, dtype=torch.int8, device="cuda")[3:]  # device spins at an odd address
+        odd.copy_(torch.from_numpy(S.reshape(-1)))
+        assert np.array_equal(inst.energy(odd), E)
+        for c in some:
+            want = _exact_energy(J, S[c], 0.75)
+            assert abs(E[c] - want) <= 4 * 2.0 ** -53 * abs(want), (N, c)
+        bad = S.copy()
+        bad[-1, -1] = 3
+        with pytest.raises(sk.SKError) as e:
+            inst.energy(bad)
+        assert e.value.status == sk.SK_ERR_INVALID_ARG and f"spin {count * N - 1} " in str(e.value)
+        inst.close()
+
+
+@pytest.mark.parametrize("low,span_fits", [(-1, True), (-45, True), (-61, True), (-62, False), (-140, False)])
+def test_energies_of_couplings_of_any_range(low, span_fits):
+    # couplings of 1 and 2^low: up to 62 bits as digits, else the direct
+    # double-precision sum (N^2/2 terms, each rounded)
+    need_gpu()
+    N, count = 70, 150
+    rng = np.random.Generator(np.random.PCG64(8))
+    J = _sym(np.where(rng.random((N, N)) < 0.5, 1.0, 2.0 ** low) * rng.choice([-1.0, 1.0], (N, N)))
+    S = inputs.initial_spins(count, N, 9)
+    inst = sk.Instance(J)
+    E = inst.energy(S)
+    inst.close()
+    total = float(np.abs(np.triu(J.astype(np.float64), 1)).sum())
+    for c in (0, count - 1):
+        want = _exact_energy(J, S[c], 1.0)
+        assert abs(E[c] - want) <= (4 * 2.0 ** -53 * abs(want) if span_fits else N * N * 2.0 ** -53 * total), c
+    zero = sk.Instance(np.zeros((N, N), dtype=np.float32))
+    assert np.array_equal(zero.energy(S), np.zeros(count))
+    zero.close()
+
+
+def test_energies_in_blocks_of_couplings_and_configurations():
+    # N = 4128: the digit slices of Gaussian couplings come in several blocks
+    # of rows, and 8200 configurations in two blocks
+    torch = need_gpu()
+    N, count = 4128, 8200
+    g = torch.Generator(device="cuda").manual_seed(3)
+    J = torch.triu(torch.randn((N, N), generator=g, device="cuda"), 1)
+    J = (J + J.T).contiguous()
+    S = (2 * torch.randint(0, 2, (count, N), generator=g, device="cuda", dtype=torch.int8) - 1).contiguous()
+    inst = sk.Instance(J)
+    E = inst.energy(S)
+    inst.close()
+    pick = [0, 127, 8063, 8064, 8199]
+    want = -0.5 * ((S[pick].double() @ J.double()) * S[pick].double()).sum(1).cpu().numpy()
+    # the reference's own rounding: ~N sums of N terms, each 2^-53 of |J| sqrt(N)
+    assert np.abs(E[pick] - want).max() <= N * np.sqrt(N) * 64 * 2.0 ** -53
