@@ -580,16 +580,17 @@ sk_status mcmcmc_run_noalloc(uint32_t N, uint32_t kind, const void* couplings, d
  * subset M of S (Eq. eq_def_rec_P), by the recursion on the first addition
  * (App. D.2; the printed recursion's normalisation differs from the process
  * by a factor that depends only on |M|, which cancels between sets of one
- * cardinality).  Computed on the device in double precision, one launch per
- * cardinality, in one of two forms:
+ * cardinality).  Computed on the device in double precision, in one of three
+ * forms:
  *   SK_SETGEN_DIRECT      every sum_{p in S \ M} P_gen(e | p) afresh,
  *                         O(n^2 2^n) work;
  *   SK_SETGEN_CUMULATIVE  the paper's cumulative table (Eq. eq_rec_set_short),
  *                         O(n 2^n) work and n 2^n doubles of device memory
  *                         (SK_ERR_OOM if they cannot be allocated);
- *   SK_SETGEN_AUTO        the cumulative form when its table can be
- *                         allocated, else the direct one.
- * The two agree to rounding (the cumulative table subtracts terms).
+ *   SK_SETGEN_AUTO        each sum as that over the six lowest elements (a
+ *                         table of 64 n doubles) plus that over the others,
+ *                         O(n 2^n) work, no table of the size of the result.
+ * They agree to rounding (the cumulative table subtracts terms).
  *   n      1..28 elements;
  *   P      n*n doubles, host, P[e*n + p] = P_gen(e | p) (finite, >= 0; the
  *          diagonal is not used);

@@ -112,12 +112,8 @@ void workspace_trim() {
         if (p) cudaMemPoolTrimTo(p, 0);
 }
 sk_status ws_alloc(void** p, size_t bytes, cudaStream_t st) {
-    *p = nullptr;
-    cudaMemPool_t pool = workspace_pool();
-    const cudaError_t e = pool ? cudaMallocFromPoolAsync(p, bytes, pool, st) : cudaErrorMemoryAllocation;
+    const cudaError_t e = sk::workspace_alloc(p, bytes, st);
     if (e == cudaSuccess) return SK_OK;
-    cudaGetLastError();
-    *p = nullptr;
     return fail(SK_ERR_OOM, "workspace of %zu bytes: %s", bytes, cudaGetErrorString(e));
 }
 
@@ -204,6 +200,16 @@ std::vector<unsigned char> graph_table(uint32_t graph, uint32_t V, uint32_t arit
 
 namespace sk {
 void set_error_message(const char* msg) { g_err = msg; }
+cudaError_t workspace_alloc(void** p, size_t bytes, cudaStream_t st) {
+    *p = nullptr;
+    cudaMemPool_t pool = workspace_pool();
+    const cudaError_t e = pool ? cudaMallocFromPoolAsync(p, bytes, pool, st) : cudaErrorMemoryAllocation;
+    if (e != cudaSuccess) {
+        cudaGetLastError();
+        *p = nullptr;
+    }
+    return e;
+}
 }  // namespace sk
 
 struct sk_instance {

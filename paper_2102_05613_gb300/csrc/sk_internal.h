@@ -306,6 +306,10 @@ size_t instance_footprint(uint32_t N, uint32_t kind);
 // outside (0, 1) or one whose smaller factor rounds to 0.
 bool root_setup(JobDev& j, uint32_t K, double p_center);
 
+// Stream-ordered workspace from the library's pool of the current device
+// (sk_capi.cu); released with cudaFreeAsync.
+cudaError_t workspace_alloc(void** p, size_t bytes, cudaStream_t st);
+
 // Sets the message sk_last_error() returns on this thread (sk_capi.cu).
 void set_error_message(const char* msg);
 

@@ -116,3 +116,21 @@ def test_energies_in_blocks_of_couplings_and_configurations():
     want = -0.5 * ((S[pick].double() @ J.double()) * S[pick].double()).sum(1).cpu().numpy()
     # the reference's own rounding: ~N sums of N terms, each 2^-53 of |J| sqrt(N)
     assert np.abs(E[pick] - want).max() <= N * np.sqrt(N) * 64 * 2.0 ** -53
+
+
+@pytest.mark.parametrize("n", [1, 2, 5, 6, 7, 10, 13, 21])
+def test_set_generation_block_form(n):
+    # below, at and above the six low elements of a block; every sum has at
+    # most 28 positive terms of relative error 2^-53 and n levels build on it
+    need_gpu()
+    rng = np.random.Generator(np.random.PCG64(n))
+    P = rng.random((n, n)) * 10.0 ** rng.integers(-3, 1, (n, n))
+    got, want = sk.set_generation(P), sk.set_generation(P, method=sk.SK_SETGEN_DIRECT)
+    assert np.all(np.abs(got - want) <= 64 * n * 2.0 ** -53 * want)
+    P[:, 0] = 0.0
+    P[0, :] = 0.0  # an element that is never generated
+    got, want = sk.set_generation(P), sk.set_generation(P, method=sk.SK_SETGEN_DIRECT)
+    assert np.all(np.abs(got - want) <= 64 * n * 2.0 ** -53 * want)
+    huge = np.full((n, n), 1e200)  # overflows to infinity, never to NaN
+    got, want = sk.set_generation(huge), sk.set_generation(huge, method=sk.SK_SETGEN_DIRECT)
+    assert np.array_equal(np.isinf(got), np.isinf(want)) and not np.isnan(got).any()
