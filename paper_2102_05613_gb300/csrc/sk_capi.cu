@@ -1432,11 +1432,49 @@ sk_status plan_batch(sk_batch* b) {
                 c.nw = tg->second >> 16;
                 c.W = tg->second & 0xFFu;
             } else {
+                // Untuned: the warps per chain that finish the class first.  A
+                // launch takes ceil(chains / (SMs x chains per CTA)) rounds and
+                // a step of a round about 1/nw + 0.05 of the one-warp step (its
+                // node passes and field update spread over the team, its
+                // barriers do not): Gaussian N = 1024, binary depth 7, us a
+                // step at nw = 1, 2, 4, 8, 16: 152 chains 66, 32, 19, 11.8, 9.8;
+                // 4096 chains 137, 67, 76, 81, 130.  One warp counts for a
+                // quarter more: with a CTA full of one-warp chains the lanes
+                // of a warp wait for its longest path (the line of 128, 4096
+                // chains: 127 in one round against 71 in two of nw = 2).  No
+                // more warps than nodes or field words to give them.
+                uint64_t total = 0;
+                uint32_t most = 1;
+                for (uint32_t i : g.second) {
+                    total += b->runs[i]->chains;
+                    const uint32_t work = std::max(b->runs[i]->job.V, b->runs[i]->inst->Npad / 4u);
+                    while (most < 16 && 32u * most < work) most <<= 1;
+                }
+                auto chains_of = [&](uint32_t nw) -> uint32_t {
+                    uint32_t ch = nw == 1 ? fitc : std::min<uint32_t>({fitc, 32u / nw, 14u}) & ~1u;
+                    if (b->W_override) ch = std::max<uint32_t>(2, std::min(ch, (b->W_override / nw) & ~1u));
+                    return ch;
+                };
                 c.nw = b->G_override >= 64 ? std::min<uint32_t>(16, b->G_override / 32) : 1u;
-                uint32_t chains = c.nw == 1 ? fitc : std::min<uint32_t>(fitc, 32 / c.nw) & ~1u;
-                if (c.nw > 1) chains = std::min<uint32_t>(chains, 14);
-                if (b->W_override) chains = std::max<uint32_t>(2, std::min(chains, (b->W_override / c.nw) & ~1u));
+                if (b->G_override == 0 && b->W_override == 0) {
+                    double best = 1e300;
+                    for (uint32_t nw = 1; nw <= most; nw <<= 1) {
+                        const uint32_t ch = chains_of(nw);
+                        if (ch < 2) break;
+                        const uint64_t per_round = static_cast<uint64_t>(sms) * ch;
+                        const double cost = static_cast<double>((total + per_round - 1) / per_round) *
+                                            (1.0 / nw + 0.05) * (nw == 1 ? 1.25 : 1.0);
+                        if (cost < best) {
+                            best = cost;
+                            c.nw = nw;
+                        }
+                    }
+                }
+                uint32_t chains = chains_of(c.nw);
                 if (chains < 2) return fail(SK_ERR_INVALID_ARG, "graph: %u warps per chain leave no room for two chains", c.nw);
+                // few chains: spread over the SMs, two per CTA at least
+                if (b->G_override == 0 && b->W_override == 0)
+                    while (chains > 2 && total <= static_cast<uint64_t>(sms) * (chains - 2)) chains -= 2;
                 c.W = chains * c.nw;
             }
             if (!sk::graph_team_ok(c.W, c.nw)) return fail(SK_ERR_INVALID_ARG, "graph layout %u warps, %u per chain", c.W, c.nw);

@@ -23,12 +23,13 @@
 //           they do when flipped in turn), the sum runs over the nodes w
 //           strictly between r and v.  Three passes over the nodes, a node
 //           per thread: x and sigma (integer work on the sites), delta (the J
-//           lookups of its path, issued four at a time), dE (the deltas along
+//           lookups of its path, issued eight at a time), dE (the deltas along
 //           its path);
 //   choice  weight ~ exp(-beta (dE_v - min)) F_v over the nodes in order
-//           (+-J: the integer table times F / 2^20; Gaussian: 2^x), each
-//           thread a contiguous chunk of nodes, a team scan of the chunk
-//           sums, the first node whose inclusive prefix exceeds u = U1 total;
+//           (+-J: the integer table times F / 2^20; Gaussian: 2^x), summed
+//           over contiguous chunks of nodes (Gaussian: 32 chunks whatever the
+//           team's size) and a scan of the chunk sums, the first node whose
+//           inclusive prefix exceeds u = U1 total;
 //   move    the chosen path's flips: h_k -= 2 sum_w sigma_w J[x_w][k] over its
 //           nodes, then each flip negates its spin in path order.
 // The oracle (sko_run_graph) defines the same chain in double precision, a
@@ -105,14 +106,15 @@ struct GMem {
     uint16_t* xs;    // [V] x_v, the site of the edge from v toward the root
     void* dl;        // [V] delta_v (H)
     void* dE;        // [V] node energy changes (H)
-    uint16_t* fx;    // [V] the move: sites flipped; during the node passes (trees) the
-                     // node's depth and its meeting depth with the root (8 bits each)
+    uint16_t* fx;    // [V] trees: the node's depth and its meeting depth with the root
+                     // (8 bits each); +-J: then the move's flipped sites
     int8_t* sg;      // [V] sigma_v
-    int8_t* fs;      // [V] the move: the spin of each flipped site before its flip
-    uint4* b0;       // block 0 of the step
+    int8_t* fs;      // [V] +-J: the move, the spin of each flipped site before its flip
+                     // (Gaussian: the move's list lies in dE, free after the weights)
+    uint4* b0;       // [2] block 0 of the steps of each parity
     void* red;       // [2][16] per-warp partial results (8 bytes each)
-    uint32_t* misc;  // [0] chosen node, [1] path length of the move, [2] the root
-    uint16_t* anc;   // [17] trees: the root's ancestor at each depth 0..depth(root)
+    uint32_t* misc;  // [0] chosen node, [1] its depths (+-J), [2 + parity] the root
+    uint16_t* anc;   // [2][20] trees: the root's ancestor at each depth 0..depth(root)
 };
 
 size_t chain_bytes(uint32_t npad, uint32_t V) {
@@ -135,9 +137,10 @@ __device__ __forceinline__ GMem chain_mem(unsigned char* base, uint32_t npad, ui
     g.fs = reinterpret_cast<int8_t*>(base + o + 15u * v16);
     unsigned char* m = base + o + 16u * v16;
     g.b0 = reinterpret_cast<uint4*>(m);
-    g.red = m + 16;
-    g.misc = reinterpret_cast<uint32_t*>(m + 16 + 256);
-    g.anc = reinterpret_cast<uint16_t*>(m + 16 + 256 + 16);
+    g.red = m + 32;
+    g.misc = reinterpret_cast<uint32_t*>(m + 32 + 256);
+    g.anc = reinterpret_cast<uint16_t*>(m + 32 + 256 + 16);
+    static_assert(32 + 256 + 16 + 2 * 20 * 2 <= kMiscBytes, "misc region");
     return g;
 }
 
@@ -204,15 +207,20 @@ __device__ __forceinline__ void graph_loop(const JobDev& jb, bool write, uint32_
     H* rmin = static_cast<H*>(gm.red);                                    // [16] warp minima
     W* rsum = reinterpret_cast<W*>(static_cast<unsigned char*>(gm.red) + 128);  // [16] warp sums
     const uint32_t nblk = (V + 2u) / 4u;  // blocks 1..nblk hold the V-1 edge sites
-    const uint32_t chunk = (V + T - 1u) / T;
+    constexpr bool kOneScan = sizeof(JT) == 4;
     uint32_t next_rec = jb.record_every ? (t0 / jb.record_every + 1u) * jb.record_every : 0u;
 
-    for (uint32_t t = t0; t < t1; ++t) {
-        // ---- draws: block 0 and the edge sites ----
-        for (uint32_t b = tid; b <= nblk; b += T) {
+    // The draws of step t: block 0, the root and the edge sites.  The edge sites
+    // are read in pass 1 only, so the next step's are drawn behind it, in the
+    // shadow of pass 2's loads, into the same array; block 0, the root and its
+    // ancestors are kept by step parity.  Thread T-1 first: the node passes
+    // leave the last threads idle where V < T.
+    auto draw = [&](uint32_t t) {
+        const uint32_t par = t & 1u;
+        for (uint32_t b = T - 1u - tid; b <= nblk; b += T) {
             const uint4 r = dev::philox4x32_10(make_uint4(b, t, chain, c3), k0, k1);
             if (b == 0u) {
-                *gm.b0 = r;
+                gm.b0[par] = r;
                 // root: tree floor(U0 V / 2^64); line the first v with
                 // P[v] > floor(U0 sum F / 2^64)
                 const unsigned long long U0 = (static_cast<unsigned long long>(r.y) << 32) | r.x;
@@ -222,7 +230,7 @@ __device__ __forceinline__ void graph_loop(const JobDev& jb, bool write, uint32_
                     // the root's ancestors by depth
                     uint32_t a = root;
                     for (uint32_t d = __ldg(&tab.dep[root]) + 1u; d-- > 0u;) {
-                        gm.anc[d] = static_cast<uint16_t>(a);
+                        gm.anc[20u * par + d] = static_cast<uint16_t>(a);
                         a = d ? tr.par(a) : 0u;
                     }
                 } else {
@@ -235,7 +243,7 @@ __device__ __forceinline__ void graph_loop(const JobDev& jb, bool write, uint32_
                     }
                     root = lo;
                 }
-                gm.misc[2] = root;
+                gm.misc[2u + par] = root;
             } else {
                 const uint32_t v0 = 4u * (b - 1u) + 1u;
                 const uint32_t w[4] = {r.x, r.y, r.z, r.w};
@@ -244,15 +252,18 @@ __device__ __forceinline__ void graph_loop(const JobDev& jb, bool write, uint32_
                     if (v0 + e < V) gm.site[v0 + e] = static_cast<uint16_t>(__umulhi(w[e], N));
             }
         }
-        if (tid == 0u) gm.misc[0] = V;  // no node chosen yet
-        team_sync(nw, team);
-        const uint4 b0 = *gm.b0;
-        const unsigned long long U0 = (static_cast<unsigned long long>(b0.y) << 32) | b0.x;
-        const unsigned long long U1 = (static_cast<unsigned long long>(b0.w) << 32) | b0.z;
+    };
+    draw(t0);
+    team_sync(nw, team);
 
-        const uint32_t root = gm.misc[2];
+    for (uint32_t t = t0; t < t1; ++t) {
+        const uint4 b0 = gm.b0[t & 1u];
+        const unsigned long long U1 = (static_cast<unsigned long long>(b0.w) << 32) | b0.z;
+        if (!kOneScan && tid == 0u) gm.misc[0] = V;  // no node chosen yet
+
+        const uint32_t root = gm.misc[2u + (t & 1u)];
         const uint32_t dr = GRAPH == 1 ? __ldg(&tab.dep[root]) : 0u;
-        const uint16_t* anc = gm.anc;
+        const uint16_t* anc = gm.anc + 20u * (t & 1u);
 
         // ---- pass 1: x_v and sigma_v ----
         for (uint32_t v = tid; v < V; v += T) {
@@ -334,6 +345,7 @@ __device__ __forceinline__ void graph_loop(const JobDev& jb, bool write, uint32_
             }
             dl[v] = static_cast<H>(2 * gm.sg[v]) * (hf[x] - static_cast<H>(2) * corr);
         }
+        if (t + 1u < t1) draw(t + 1u);
         team_sync(nw, team);
 
         // ---- pass 3: dE_v = sum of delta over the path's nodes after r ----
@@ -362,12 +374,11 @@ __device__ __forceinline__ void graph_loop(const JobDev& jb, bool write, uint32_
         }
         team_sync(nw, team);
 
-        // ---- choice: weights over contiguous node chunks, team scan ----
-        const uint32_t v0 = tid * chunk, v1 = min(V, v0 + chunk);
+        // ---- choice ----
         H mloc = H(0);
-        for (uint32_t v = v0; v < v1; ++v)
+        for (uint32_t v = tid; v < V; v += T)
             if (__ldg(&tab.F[v]) && dE[v] < mloc) mloc = dE[v];
-        mloc = step::gmin<false>(g, mloc);
+        mloc = step::gmin<true>(g, mloc);
         if (nw > 1u) {
             if (lane == 0u) rmin[wt] = mloc;
             team_sync(nw, team);
@@ -389,64 +400,101 @@ __device__ __forceinline__ void graph_loop(const JobDev& jb, bool write, uint32_
                 return dev::pow2(fmaf(nbl2, dE[v] - m, __ldg(&tab.lg[v])));
             }
         };
-        W lsum = W(0);
-        for (uint32_t v = v0; v < v1; ++v) lsum += node_w(v);
-        const W incl = step::gscan(g, lsum);
-        const W wtot = __shfl_sync(kFull, incl, 31);
-        W excl = W(0), total = wtot;
-        if (nw > 1u) {
-            if (lane == 31u) rsum[wt] = wtot;
+        uint32_t jsel = V;
+        uint32_t jdep = 0;  // trees: its depth and meeting depth
+        if constexpr (kOneScan) {
+            // Gaussian weights: a node per thread into shared memory, then every
+            // warp of the team takes the same scan -- lane l the nodes l c ..
+            // l c + c - 1, c = ceil(V / 32), in order, then the lanes -- so that
+            // the fp32 sums, and with them the trajectory, do not depend on the
+            // warps per chain, and no barrier stands between the scan and the
+            // move.  (Before, each thread summed its own chunk and the warps'
+            // totals met at two more barriers.)
+            float* wv = reinterpret_cast<float*>(dl);
+            for (uint32_t v = tid; v < V; v += T) wv[v] = node_w(v);
             team_sync(nw, team);
-            W run = W(0);
-            for (uint32_t w = 0; w < nw; ++w) {
-                if (w == wt) excl = run;
-                run += rsum[w];
-            }
-            total = run;
-        }
-        W u;
-        if constexpr (sizeof(JT) == 1) {
-            u = __umul64hi(U1, total);
-        } else {
-            u = static_cast<float>(U1 >> 40) * 0x1p-24f * total;
+            const uint32_t chunk = (V + 31u) / 32u, v0 = lane * chunk, v1 = min(V, v0 + chunk);
+            W lsum = W(0);
+            for (uint32_t v = v0; v < v1; ++v) lsum += wv[v];
+            const W incl = step::gscan(g, lsum);
+            const W total = __shfl_sync(kFull, incl, 31);
+            W u = static_cast<float>(U1 >> 40) * 0x1p-24f * total;
             if (u >= total) u = nextafterf(total, 0.0f);
-        }
-        // the warp whose range [excl, excl + wtot) holds u: its first lane
-        // whose prefix exceeds u searches its chunk (else, a rounding guard,
-        // its last positive weight)
-        if (wtot > W(0) && u >= excl && u < excl + wtot) {
-            const unsigned ball = __ballot_sync(kFull, excl + incl > u);
-            const int L = ball ? __ffs(ball) - 1 : 31;
-            if (static_cast<int>(lane) == L) {
-                W run = excl + (incl - lsum);
+            if (total > W(0) && u < total) {
+                const unsigned ball = __ballot_sync(kFull, incl > u);
+                const int L = ball ? __ffs(ball) - 1 : 31;
                 int found = -1, last = -1;
-                for (uint32_t v = v0; v < v1; ++v) {
-                    const W x = node_w(v);
-                    if (x > W(0)) {
-                        last = static_cast<int>(v);
-                        if (found < 0) {
-                            run += x;
-                            if (run > u) found = static_cast<int>(v);
+                if (static_cast<int>(lane) == L) {
+                    // its first node whose prefix exceeds u (else, a rounding
+                    // guard, its last positive weight)
+                    W run = incl - lsum;
+                    for (uint32_t v = v0; v < v1; ++v) {
+                        const W x = wv[v];
+                        if (x > W(0)) {
+                            last = static_cast<int>(v);
+                            if (found < 0) {
+                                run += x;
+                                if (run > u) found = static_cast<int>(v);
+                            }
                         }
                     }
                 }
-                const uint32_t js = static_cast<uint32_t>(found >= 0 ? found : last);
-                gm.misc[0] = js;
-                if constexpr (GRAPH == 1) gm.misc[3] = js < V ? gm.fx[js] : 0u;
+                jsel = static_cast<uint32_t>(__shfl_sync(kFull, found >= 0 ? found : last, L));
             }
+            if (jsel >= V) jsel = root;  // no positive weight found (cannot happen for finite fields): stay
+            if constexpr (GRAPH == 1) jdep = gm.fx[jsel];
+        } else {
+            // +-J weights (64 bits, exact in any order): contiguous node chunks
+            // per thread, a team scan of the chunk sums
+            const uint32_t chunk = (V + T - 1u) / T;
+            const uint32_t v0 = tid * chunk, v1 = min(V, v0 + chunk);
+            W lsum = W(0);
+            for (uint32_t v = v0; v < v1; ++v) lsum += node_w(v);
+            const W incl = step::gscan(g, lsum);
+            const W wtot = __shfl_sync(kFull, incl, 31);
+            W excl = W(0), total = wtot;
+            if (nw > 1u) {
+                if (lane == 31u) rsum[wt] = wtot;
+                team_sync(nw, team);
+                W run = W(0);
+                for (uint32_t w = 0; w < nw; ++w) {
+                    if (w == wt) excl = run;
+                    run += rsum[w];
+                }
+                total = run;
+            }
+            const W u = __umul64hi(U1, total);
+            // the warp whose range [excl, excl + wtot) holds u: its first lane
+            // whose prefix exceeds u searches its chunk
+            if (wtot > W(0) && u >= excl && u < excl + wtot) {
+                const unsigned ball = __ballot_sync(kFull, excl + incl > u);
+                const int L = ball ? __ffs(ball) - 1 : 31;
+                if (static_cast<int>(lane) == L) {
+                    W run = excl + (incl - lsum);
+                    uint32_t js = V;
+                    for (uint32_t v = v0; v < v1 && js == V; ++v) {
+                        run += node_w(v);
+                        if (run > u) js = v;
+                    }
+                    gm.misc[0] = js;
+                    if constexpr (GRAPH == 1) gm.misc[1] = js < V ? gm.fx[js] : 0u;
+                }
+            }
+            team_sync(nw, team);
+            jsel = gm.misc[0];
+            if (jsel >= V) jsel = root;
+            if constexpr (GRAPH == 1) jdep = jsel == root ? (dr | (dr << 8)) : gm.misc[1];
         }
-        team_sync(nw, team);
-        uint32_t jsel = gm.misc[0];
-        if (jsel >= V) jsel = root;  // no positive weight found (cannot happen for finite fields): stay
 
         // ---- move: the chosen path's flips ----
         // the path's nodes after r, one per thread: the ancestors of r up to
         // the meeting node, then jsel and its ancestors below it (the order
         // of the flips does not matter: the signs are those of the path)
+        uint16_t* lx = kOneScan ? reinterpret_cast<uint16_t*>(dE) : gm.fx;
+        int8_t* ls = kOneScan ? reinterpret_cast<int8_t*>(dE) + 2u * V : gm.fs;
         uint32_t n;
         if constexpr (GRAPH == 1) {
-            const uint32_t dd = jsel == root ? (dr | (dr << 8)) : gm.misc[3];
-            const uint32_t dj = dd & 0xFFu, dm = dd >> 8;
+            const uint32_t dj = jdep & 0xFFu, dm = jdep >> 8;
             const uint32_t na = dr - dm;
             n = na + dj - dm;
             for (uint32_t i = tid; i < n; i += T) {
@@ -457,8 +505,8 @@ __device__ __forceinline__ void graph_loop(const JobDev& jb, bool write, uint32_
                     w = jsel;
                     for (uint32_t q = na; q < i; ++q) w = tr.par(w);
                 }
-                gm.fx[i] = gm.xs[w];
-                gm.fs[i] = gm.sg[w];
+                lx[i] = gm.xs[w];
+                ls[i] = gm.sg[w];
             }
         } else {
             const uint32_t lo = min(root, jsel), hi = max(root, jsel);
@@ -466,13 +514,14 @@ __device__ __forceinline__ void graph_loop(const JobDev& jb, bool write, uint32_
             for (uint32_t i = tid; i < n; i += T) {
                 const uint32_t w = lo + 1u + i;  // the nodes lo+1..hi: one of them is r, the other end jsel
                 const uint32_t ww = jsel > root ? w : w - 1u;
-                gm.fx[i] = gm.xs[ww];
-                gm.fs[i] = gm.sg[ww];
+                lx[i] = gm.xs[ww];
+                ls[i] = gm.sg[ww];
             }
         }
         team_sync(nw, team);
         // fields: h_k -= 2 sum_i fs_i J[fx_i][k], four elements per thread,
-        // the rows' loads issued four flips at a time
+        // the rows' loads issued eight flips at a time (a binary tree of depth 7 moves ~10:
+        // two round trips to L2 where four at a time took three)
         for (uint32_t k = 4u * tid; k < npad; k += 4u * T) {
             const JT* col = Jg + k;
             if constexpr (sizeof(JT) == 1) {
@@ -484,25 +533,25 @@ __device__ __forceinline__ void graph_loop(const JobDev& jb, bool write, uint32_
                     hv.w -= c * dev::sbyte(j, 3);
                 };
                 uint32_t i = 0;
-                for (; i + 4u <= n; i += 4u) {
-                    uint32_t j[4];
+                for (; i + 8u <= n; i += 8u) {
+                    uint32_t j[8];
 #pragma unroll
-                    for (int q = 0; q < 4; ++q)
-                        j[q] = __ldg(reinterpret_cast<const unsigned int*>(col + static_cast<size_t>(gm.fx[i + q]) * npad));
+                    for (int q = 0; q < 8; ++q)
+                        j[q] = __ldg(reinterpret_cast<const unsigned int*>(col + static_cast<size_t>(lx[i + q]) * npad));
 #pragma unroll
-                    for (int q = 0; q < 4; ++q) upd(j[q], 2 * gm.fs[i + q]);
+                    for (int q = 0; q < 8; ++q) upd(j[q], 2 * ls[i + q]);
                 }
-                if (i < n) {  // the last n - i < 4 rows together
+                if (i < n) {  // the last n - i < 8 rows together
                     const uint32_t r = n - i;
-                    uint32_t j[3];
+                    uint32_t j[7];
 #pragma unroll
-                    for (uint32_t q = 0; q < 3u; ++q)
+                    for (uint32_t q = 0; q < 7u; ++q)
                         j[q] = q < r ? __ldg(reinterpret_cast<const unsigned int*>(
-                                           col + static_cast<size_t>(gm.fx[i + q]) * npad))
+                                           col + static_cast<size_t>(lx[i + q]) * npad))
                                      : 0u;
 #pragma unroll
-                    for (uint32_t q = 0; q < 3u; ++q)
-                        if (q < r) upd(j[q], 2 * gm.fs[i + q]);
+                    for (uint32_t q = 0; q < 7u; ++q)
+                        if (q < r) upd(j[q], 2 * ls[i + q]);
                 }
                 *reinterpret_cast<int4*>(hf + k) = hv;
             } else {
@@ -514,24 +563,24 @@ __device__ __forceinline__ void graph_loop(const JobDev& jb, bool write, uint32_
                     hv.w = fmaf(-c, j.w, hv.w);
                 };
                 uint32_t i = 0;
-                for (; i + 4u <= n; i += 4u) {
-                    float4 j[4];
+                for (; i + 8u <= n; i += 8u) {
+                    float4 j[8];
 #pragma unroll
-                    for (int q = 0; q < 4; ++q)
-                        j[q] = __ldg(reinterpret_cast<const float4*>(col + static_cast<size_t>(gm.fx[i + q]) * npad));
+                    for (int q = 0; q < 8; ++q)
+                        j[q] = __ldg(reinterpret_cast<const float4*>(col + static_cast<size_t>(lx[i + q]) * npad));
 #pragma unroll
-                    for (int q = 0; q < 4; ++q) upd(j[q], static_cast<float>(2 * gm.fs[i + q]));
+                    for (int q = 0; q < 8; ++q) upd(j[q], static_cast<float>(2 * ls[i + q]));
                 }
-                if (i < n) {  // the last n - i < 4 rows together
+                if (i < n) {  // the last n - i < 8 rows together
                     const uint32_t r = n - i;
-                    float4 j[3];
+                    float4 j[7];
 #pragma unroll
-                    for (uint32_t q = 0; q < 3u; ++q)
-                        j[q] = q < r ? __ldg(reinterpret_cast<const float4*>(col + static_cast<size_t>(gm.fx[i + q]) * npad))
+                    for (uint32_t q = 0; q < 7u; ++q)
+                        j[q] = q < r ? __ldg(reinterpret_cast<const float4*>(col + static_cast<size_t>(lx[i + q]) * npad))
                                      : make_float4(0.f, 0.f, 0.f, 0.f);
 #pragma unroll
-                    for (uint32_t q = 0; q < 3u; ++q)
-                        if (q < r) upd(j[q], static_cast<float>(2 * gm.fs[i + q]));
+                    for (uint32_t q = 0; q < 7u; ++q)
+                        if (q < r) upd(j[q], static_cast<float>(2 * ls[i + q]));
                 }
                 *reinterpret_cast<float4*>(hf + k) = hv;
             }
@@ -540,11 +589,11 @@ __device__ __forceinline__ void graph_loop(const JobDev& jb, bool write, uint32_
         // occurs an odd number of times; the state changed iff one does
         bool odd = false;
         for (uint32_t i = tid; i < n; i += T) {
-            const uint32_t x = gm.fx[i];
+            const uint32_t x = lx[i];
             bool first = true;
             uint32_t c = 0;
             for (uint32_t j = 0; j < n; ++j) {
-                const bool eq = gm.fx[j] == x;
+                const bool eq = lx[j] == x;
                 c += eq ? 1u : 0u;
                 first = first && !(eq && j < i);
             }
@@ -557,7 +606,7 @@ __device__ __forceinline__ void graph_loop(const JobDev& jb, bool write, uint32_
         acc += changed ? 1u : 0u;
         n_flips += n;
         if (t < trace_end && tid == 0u) jb.trace[static_cast<size_t>(chain) * jb.trace_steps + t] = static_cast<int32_t>(jsel);
-        team_sync(nw, team);
+        if (nw == 1u) __syncwarp();  // (a team of several warps has just met in team_any)
         if (t + 1u == next_rec) {
             step::record<JT, 0, 1, 32, false>(jb, write && wt == 0u, chain, next_rec / jb.record_every - 1u, S, hf,
                                               partner_off, acc, next_rec);

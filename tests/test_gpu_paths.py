@@ -134,3 +134,37 @@ def test_set_generation_block_form(n):
     huge = np.full((n, n), 1e200)  # overflows to infinity, never to NaN
     got, want = sk.set_generation(huge), sk.set_generation(huge, method=sk.SK_SETGEN_DIRECT)
     assert np.array_equal(np.isinf(got), np.isinf(want)) and not np.isnan(got).any()
+
+
+@pytest.mark.parametrize("graph,arity,depth,L,N,chains", [
+    (sk.SK_GRAPH_TREE, 2, 7, 0, 200, 5),     # 255 nodes: chunks of 8, ragged last lane
+    (sk.SK_GRAPH_TREE, 3, 2, 0, 64, 3),      # 13 nodes: fewer than lanes
+    (sk.SK_GRAPH_TREE, 16, 2, 0, 1000, 2),   # 273 nodes, odd chunks
+    (sk.SK_GRAPH_LINE, 0, 0, 128, 130, 4),   # nodes of factor 0
+    (sk.SK_GRAPH_LINE, 0, 0, 33, 40, 1),
+])
+def test_graph_results_do_not_depend_on_the_warps_per_chain(graph, arity, depth, L, N, chains):
+    # Gaussian couplings: the weights are summed in one order whatever the team
+    # (and the default picks a team by the number of chains)
+    need_gpu()
+    J = inputs.couplings_gauss(N, 31)
+    init = inputs.initial_spins(chains, N, 32)
+    outs = []
+    for lanes in (0, 32, 64, 128, 256, 512):
+        inst = sk.Instance(J)
+        run = sk.Run(inst, chains=chains, K=1, beta=1.3, seed=33, record_every=40, max_records=3, init=init,
+                     trace_chains=chains, trace_steps=120, graph=graph, arity=arity, depth=depth, line_nodes=L)
+        b = sk.Batch([run])
+        b.set_layout(lanes=lanes)
+        b.advance(41)
+        b.advance(79)
+        E, q, acc = run.observables()
+        outs.append((run.trace(), E, q, acc) + run.state(fields=True))
+        b.close(); run.close(); inst.close()
+    for o in outs[1:]:
+        assert all(np.array_equal(x, y) for x, y in zip(outs[0], o))
+    for c in range(chains):
+        r = oracle.replay_graph(J, outs[0][0][c], graph=oracle.TREE if graph == sk.SK_GRAPH_TREE else oracle.LINE,
+                                arity=arity, depth=depth, line_nodes=L, beta=1.3, seed=33, chain=c, init=init[c],
+                                tol=1e-4)
+        assert r["bad"] == 0, (c, r)
