@@ -415,7 +415,11 @@ sk_status mcmcmc_batch_autotune(sk_batch* b, uint32_t trial_steps, uint32_t* war
  *   lanes    lanes per chain, 4, 8, 16 or 32 (32/lanes chains share a warp),
  *            raised to the fewest a class's K allows (each lane draws up to
  *            4 Philox blocks of 4 proposals: see below);
- *            0 = default (whole-warp chains, 32 lanes); a value that
+ *            0 = default: whole-warp chains (32 lanes), or for star classes
+ *            the team layout of 2 or 4 warps per chain (64 / 128 lanes below)
+ *            where the batch's chains are few enough to run in one round of
+ *            its CTAs, and for graph classes the warps per chain that finish
+ *            the class's chains first; a value that
  *            leaves no room for one warp's chains in a CTA's shared memory
  *            is raised until they fit.  Kernels exist
  *            for 1 block per lane at every width, 2 blocks at 8, 16 and 32
@@ -429,7 +433,7 @@ sk_status mcmcmc_batch_autotune(sk_batch* b, uint32_t trial_steps, uint32_t* war
  *            the class has one chain, else two (overlap pairs share a CTA);
  *            MCMCMC with K <= 32 x warps per chain, or Metropolis, and no
  *            node-weighted records (other classes fall back to 32 lanes).
- *            +-J trajectories are those of the warp layouts bit for bit;
+ *            Trajectories are those of 32 lanes bit for bit;
  *   staging  0 = default (rows through L1), 1 = the next step's row of J is
  *            staged in shared memory by TMA (two row buffers per chain),
  *            2 = rows are read through L1 (no buffers, so more chains fit in

@@ -1380,6 +1380,43 @@ bool plan_team_class(const sk_batch* b, const std::vector<uint32_t>& idx, uint32
     return true;
 }
 
+// Warps per chain of the team layout a star class gets without being asked
+// for a layout (0: the warp layouts).  Results are the same either way.  A
+// team shortens a chain's step, so it is taken where the batch's chains are so
+// few that all are in flight in one round of the class's CTAs.  ns a step, one
+// warp / 2 warps / 4 warps per chain, one chain and 304 chains, N = 512 (2048):
+//   Metropolis, Gaussian  287 / 190 / 189;  309 / 206 / 210 (356 / 285 / 230)
+//   K = 8, Gaussian       843 / 733 / 748;  886 / 792 / 788 (1259 / 988 / 860)
+//   K = 64                1221 / 943 / 919;  1278 / 1001 / 983 (1895 / 1353 / 1130)
+//   K = 128               1254 / - / 945;  1295 / - / 1010 (2016 / - / 1194)
+// and beyond: 608 chains K = 64 1283 / 1043 / 1949 (two rounds), 1216 chains
+// Metropolis 324 / 240 / 449.  +-J runs whose weight
+// table fits the shared copy have a one-warp loop of their own, the faster one
+// up to K = 32 (K = 8 512 / 685, K = 32 553 / 657; K = 64 819 / 705).
+uint32_t default_team(const sk_batch* b, const std::vector<uint32_t>& idx, int sms) {
+    const sk_run* r0 = b->runs[idx[0]];
+    if (run_nw(r0) || r0->p.graph) return 0;
+    uint64_t total = 0;  // star chains of the whole batch: its classes share the SMs
+    for (const sk_run* r : b->runs)
+        if (!r->p.graph) total += r->chains;
+    uint32_t K = 1, npad = 0;
+    bool short_tables = r0->inst->kind == SK_J_PM1, single = true;
+    for (uint32_t i : idx) {
+        const sk_run* r = b->runs[i];
+        K = std::max(K, r->p.K);
+        npad = std::max(npad, r->inst->Npad);
+        short_tables = short_tables && r->wlen <= 64u;
+        single = single && r->chains == 1;
+    }
+    if (K > 128u || (short_tables && r0->p.rule == SK_RULE_MCMCMC && K <= 32u)) return 0;
+    const uint32_t per_cta = single ? 1u : 2u;
+    const uint64_t s = static_cast<uint64_t>(sms);
+    // 4 warps: one CTA per SM; 2 warps: two (Metropolis, fewer registers: four)
+    if (total <= per_cta * s && (K > 64u || npad >= 1024u)) return 4;
+    if (K <= 64u && total <= (r0->p.rule == SK_RULE_METROPOLIS ? 4u : 2u) * per_cta * s) return 2;
+    return 0;
+}
+
 // Work items of the batch, grouped by launch class, each class with its own
 // lanes per chain and warps per CTA: the autotuned or forced values, else
 // the fewest lanes K allows (whole-warp chains for runs of few chains, where
@@ -1527,7 +1564,9 @@ sk_status plan_batch(sk_batch* b) {
            // forced by mcmcmc_batch_set_layout with 64 or more lanes
             auto tt = b->tuned.find(c.key);
             const bool tuned_t = tt != b->tuned.end() && (tt->second >> 24) == 0 && ((tt->second >> 8) & 0xFFu) >= 64;
-            const uint32_t lanes = tuned_t ? ((tt->second >> 8) & 0xFFu) : (tt == b->tuned.end() ? b->G_override : 0u);
+            uint32_t lanes = tuned_t ? ((tt->second >> 8) & 0xFFu) : (tt == b->tuned.end() ? b->G_override : 0u);
+            if (tt == b->tuned.end() && !b->G_override && !b->S_override && !b->W_override && !b->C_override)
+                lanes = 32u * default_team(b, g.second, sms);
             if (lanes >= 64 &&
                 plan_team_class(b, g.second, lanes >= 128 ? 4u : 2u, tuned_t ? (tt->second & 0xFFu) : 0u, c)) {
                 const int occ = sk::team_occupancy(c.kind, c.rule, c.team, c.W, c.per_chain);

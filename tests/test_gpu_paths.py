@@ -168,3 +168,32 @@ def test_graph_results_do_not_depend_on_the_warps_per_chain(graph, arity, depth,
                                 arity=arity, depth=depth, line_nodes=L, beta=1.3, seed=33, chain=c, init=init[c],
                                 tol=1e-4)
         assert r["bad"] == 0, (c, r)
+
+
+@pytest.mark.parametrize("K,rule,p_center,lanes", [(1, 0, 0.0, 64), (5, 0, 0.0, 128), (32, 0, 0.2, 64), (33, 0, 0.0, 64),
+                                                   (64, 0, 0.0, 64), (65, 0, 0.0, 128), (100, 0, 0.05, 128),
+                                                   (128, 0, 0.0, 128), (1, 1, 0.0, 64), (1, 1, 0.0, 128)])
+@pytest.mark.parametrize("N,chains", [(96, 3), (515, 1)])
+def test_team_results_are_those_of_one_warp_per_chain(K, rule, p_center, lanes, N, chains):
+    # Gaussian couplings: a team sums the weights in the one-warp order, so the
+    # layouts (and the default, which picks one by the number of chains) agree
+    # bit for bit; advances of ragged lengths cross the draws' batches
+    need_gpu()
+    J = inputs.couplings_gauss(N, 41)
+    init = inputs.initial_spins(chains, N, 42)
+    outs = []
+    for lay in (32, lanes, 0):
+        inst = sk.Instance(J)
+        run = sk.Run(inst, chains=chains, K=K, rule=rule, beta=1.2, seed=43, record_every=50, max_records=6, init=init,
+                     trace_chains=chains, trace_steps=300, p_center=p_center)
+        b = sk.Batch([run])
+        b.set_layout(lanes=lay)
+        if lay != 0:
+            assert b.classes()[0][1] == lay
+        for n in (1, 32, 67, 200):
+            b.advance(n)
+        E, q, acc = run.observables()
+        outs.append((run.trace(), E, q, acc) + run.state(fields=True) + run.counters())
+        b.close(); run.close(); inst.close()
+    for o in outs[1:]:
+        assert all(np.array_equal(x, y) for x, y in zip(outs[0], o))
