@@ -203,7 +203,7 @@ int occupancy_cluster_gauss(uint32_t rule, uint32_t nb, uint32_t C, uint32_t W, 
 // memory per chain: spins, fields, the site ring, T block-0 buffers and the
 // team's exchange words (minima, the slots' weights).  launch_team runs the items of one class.
 inline size_t team_chain_bytes(uint32_t npad, uint32_t T) {
-    return ((size_t)5 * npad + 1024u * T + 16u + 256u * T + 127u) & ~(size_t)127;
+    return ((size_t)5 * npad + 1024u * T + 32u + 256u * T + 127u) & ~(size_t)127;
 }
 inline bool team_ok(uint32_t rule, uint32_t K, uint32_t T) {
     return (T == 2 || T == 4) && (rule == 1 || (K >= 1 && K <= 32u * T));
