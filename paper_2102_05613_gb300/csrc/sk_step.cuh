@@ -227,6 +227,30 @@ __device__ __forceinline__ uint32_t site_of(const uint32_t (&sp)[2 * NB], int k)
     return (sp[k >> 1] >> (16 * (k & 1))) & 0xFFFFu;
 }
 
+// Entry e (0..3, known at run time) of the two packed words of one block.
+__device__ __forceinline__ uint32_t site_pick(uint32_t w0, uint32_t w1, int e) {
+    return (((e & 2) ? w1 : w0) >> (16 * (e & 1))) & 0xFFFFu;
+}
+// The first of a lane's four weights whose prefix run + x[0] + .. exceeds u;
+// failing that (a rounding guard) its last positive one, -1 if there is none.  The prefixes are
+// taken one after the other, the comparisons side by side: a weight of 0 adds
+// nothing and is not taken, so this is the search that stops at the first.
+// Taken where registers allow (the 128-register variant, teams): in the
+// throughput variants it costs 8 % (65,536 chains, N = 512, K = 128, 80
+// registers: 36.7 -> 39.8 us a step).
+template <typename W>
+__device__ __forceinline__ int first_past(const W (&x)[4], W run, W u) {
+    uint32_t past = 0, pos = 0;
+#pragma unroll
+    for (int e = 0; e < 4; ++e) {
+        run += x[e];
+        const bool p = x[e] > W(0);
+        pos |= p ? 1u << e : 0u;
+        past |= p && run > u ? 1u << e : 0u;
+    }
+    return past ? __ffs(static_cast<int>(past)) - 1 : 31 - __clz(static_cast<int>(pos));
+}
+
 // h_k -= c1 J[x1][k] + c2 J[x2][k] for k < Npad (c2 = 0: one flip); lane gl
 // owns elements 4 gl + 4 G v.  r1 is the staged row (shared memory) when
 // STAGED, else a row of J in global memory; r2 is global and read only when
@@ -583,6 +607,11 @@ __device__ __forceinline__ void chain_loop(const JobDev& jb, bool write, uint32_
     // and their lookups in the owning lanes of every group) and with one slot
     // per lane (one weight)
     constexpr bool KEEPXS = KEEPW || NB == 2 || SPL1;
+    // the forms that cost registers or code but fewer dependent instructions
+    // (one chain, ns a step: Gaussian N = 512, K = 128 1251 -> 1172, K = 256
+    // 1552 -> 1435; the uneven fused batch 3 %): not in the throughput
+    // variants, nor in the +-J loop of one slot per lane (533 -> 549 at K = 8)
+    constexpr bool LEAN = KEEPW && !(SPL1 && sizeof(JT) == 1);
     constexpr int NQ = SPL1 ? 1 : 4 * NB;  // slots per lane
     constexpr int SCANL = SPL1 ? (4 * SL < G ? 4 * SL : G) : (SL > 0 ? SL : 1);
     const Grp<G> g;
@@ -842,7 +871,9 @@ __device__ __forceinline__ void chain_loop(const JobDev& jb, bool write, uint32_
                     u = __umul64hi(U1, total);
                 } else {
                     u = static_cast<float>(U1 >> 40) * 0x1p-24f * total;
-                    if (u >= total) u = nextafterf(total, 0.0f);
+                    // (at most the float below the total, which is positive)
+                    if constexpr (LEAN) u = fminf(u, __uint_as_float(__float_as_uint(total) - 1u));
+                    else if (u >= total) u = nextafterf(total, 0.0f);
                 }
                 // first slot whose inclusive prefix exceeds u; the owning
                 // lane finds its entry (else, a rounding guard, its last
@@ -908,25 +939,38 @@ __device__ __forceinline__ void chain_loop(const JobDev& jb, bool write, uint32_
                         W mine = 0;
 #pragma unroll
                         for (int e = 0; e < 4; ++e) mine += x[e];
-                        W run = bse + (inc - mine);
-                        int my_e = -1, last_pos = -1;
+                        uint32_t my_site = 0;
+                        int my_e = -1;
+                        if constexpr (LEAN) {
+                            my_e = first_past(x, bse + (inc - mine), u);
+                            uint32_t sw0 = site[0], sw1 = site[1];
 #pragma unroll
-                        for (int e = 0; e < 4; ++e) {
-                            if (x[e] > W(0)) {
-                                last_pos = e;
-                                if (my_e < 0) {
-                                    run += x[e];
-                                    if (run > u) my_e = e;
+                            for (int q = 1; q < NB; ++q)
+                                if (q == qf) {
+                                    sw0 = site[2 * q];
+                                    sw1 = site[2 * q + 1];
+                                }
+                            if (my_e >= 0) my_site = site_pick(sw0, sw1, my_e);
+                        } else {
+                            W run = bse + (inc - mine);
+                            int last_pos = -1;
+#pragma unroll
+                            for (int e = 0; e < 4; ++e) {
+                                if (x[e] > W(0)) {
+                                    last_pos = e;
+                                    if (my_e < 0) {
+                                        run += x[e];
+                                        if (run > u) my_e = e;
+                                    }
                                 }
                             }
+                            if (my_e < 0) my_e = last_pos;
+#pragma unroll
+                            for (int q = 0; q < NB; ++q)
+#pragma unroll
+                                for (int e = 0; e < 4; ++e)
+                                    if (q == qf && e == my_e) my_site = site_of<NB>(site, 4 * q + e);
                         }
-                        if (my_e < 0) my_e = last_pos;
-                        uint32_t my_site = 0;
-#pragma unroll
-                        for (int q = 0; q < NB; ++q)
-#pragma unroll
-                            for (int e = 0; e < 4; ++e)
-                                if (q == qf && e == my_e) my_site = site_of<NB>(site, 4 * q + e);
                         const uint32_t packed = gshfl(g, (my_site << 2) | static_cast<uint32_t>(my_e & 3), L);
                         sel_site = packed >> 2;
                         sel_d = 4 * G * qf + 4 * L + static_cast<int>(packed & 3u) + 1;
@@ -951,23 +995,29 @@ __device__ __forceinline__ void chain_loop(const JobDev& jb, bool write, uint32_
                                 x[e] = slot_w(4 * q + e);
                             mine += x[e];
                         }
-                        W run = base + (incl[q] - mine);
-                        int my_e = -1, last_pos = -1;
+                        uint32_t my_site = 0;
+                        int my_e = -1;
+                        if constexpr (LEAN) {
+                            my_e = first_past(x, base + (incl[q] - mine), u);
+                            if (my_e >= 0) my_site = site_pick(site[2 * q], site[2 * q + 1], my_e);
+                        } else {
+                            W run = base + (incl[q] - mine);
+                            int last_pos = -1;
 #pragma unroll
-                        for (int e = 0; e < 4; ++e) {
-                            if (x[e] > W(0)) {
-                                last_pos = e;
-                                if (my_e < 0) {
-                                    run += x[e];
-                                    if (run > u) my_e = e;
+                            for (int e = 0; e < 4; ++e) {
+                                if (x[e] > W(0)) {
+                                    last_pos = e;
+                                    if (my_e < 0) {
+                                        run += x[e];
+                                        if (run > u) my_e = e;
+                                    }
                                 }
                             }
-                        }
-                        if (my_e < 0) my_e = last_pos;
-                        uint32_t my_site = 0;
+                            if (my_e < 0) my_e = last_pos;
 #pragma unroll
-                        for (int e = 0; e < 4; ++e)
-                            if (e == my_e) my_site = site_of<NB>(site, 4 * q + e);
+                            for (int e = 0; e < 4; ++e)
+                                if (e == my_e) my_site = site_of<NB>(site, 4 * q + e);
+                        }
                         const uint32_t packed = gshfl(g, (my_site << 2) | static_cast<uint32_t>(my_e & 3), L);
                         sel_site = packed >> 2;
                         sel_d = 4 * G * q + 4 * L + static_cast<int>(packed & 3u) + 1;
@@ -1002,14 +1052,17 @@ __device__ __forceinline__ void chain_loop(const JobDev& jb, bool write, uint32_
                 // chunks in the RCH instantiation (rows whose per-lane share is
                 // not a whole number of unrolled passes), else the unrolled loop
                 constexpr bool CHUNKED = UNROLL >= 8 && (RULE == 0 || RCH);
-                if (x1_staged)
-                    update_fields<JT, STAGED, G, UNROLL, CHUNKED, RULE == 0>(hf, rowA, Jrow(x2), c1, c2, npad, g.gl);
+                // (LEAN: one form for a row a or another first row; with 80
+                // registers the two forms are 12 % faster)
+                if (x1_staged || (LEAN && !STAGED))
+                    update_fields<JT, STAGED, G, UNROLL, CHUNKED, RULE == 0>(hf, LEAN && !STAGED ? Jrow(x1) : rowA, Jrow(x2), c1, c2,
+                                                                              npad, g.gl);
                 else
                     update_fields<JT, false, G, UNROLL, CHUNKED, false>(hf, Jrow(x1), nullptr, c1, 0, npad, g.gl);
                 __syncwarp(g.mask);
                 if (g.gl == 0) {
-                    S[x1] = static_cast<int8_t>(-S[x1]);
-                    if (nflip == 2) S[x2] = static_cast<int8_t>(-S[x2]);
+                    S[x1] = static_cast<int8_t>(LEAN ? (c1 > 0 ? -1 : 1) : -S[x1]);
+                    if (nflip == 2) S[x2] = static_cast<int8_t>(LEAN ? (c2 > 0 ? -1 : 1) : -S[x2]);
                 }
                 acc += 1u;
             }

@@ -102,29 +102,6 @@ __device__ __forceinline__ uint32_t get_weights4(const unsigned long long* p, un
     return neg;
 }
 
-// Entry e (0..3, known at run time) of the two packed words of one block.
-__device__ __forceinline__ uint32_t site_pick(uint32_t w0, uint32_t w1, int e) {
-    return (((e & 2) ? w1 : w0) >> (16 * (e & 1))) & 0xFFFFu;
-}
-// The first of a lane's four weights whose prefix run + x[0] + .. exceeds u;
-// failing that (a rounding guard) its last positive one, -1 if there is none.  The prefixes are
-// taken one after the other, the comparisons side by side: a weight of 0 adds
-// nothing and is not taken, so this is the search that stops at the first.
-// (In the warp layouts' throughput kernels the same form cost 8 %: 36.7 -> 39.8
-// us a step of 65,536 chains, N = 512, K = 128, by registers.)
-template <typename W>
-__device__ __forceinline__ int first_past(const W (&x)[4], W run, W u) {
-    uint32_t past = 0, pos = 0;
-#pragma unroll
-    for (int e = 0; e < 4; ++e) {
-        run += x[e];
-        const bool p = x[e] > W(0);
-        pos |= p ? 1u << e : 0u;
-        past |= p && run > u ? 1u << e : 0u;
-    }
-    return past ? __ffs(static_cast<int>(past)) - 1 : 31 - __clz(static_cast<int>(pos));
-}
-
 __device__ __forceinline__ void team_sync(int id, int nthreads) {
     asm volatile("bar.sync %0, %1;" ::"r"(id), "r"(nthreads) : "memory");
 }
@@ -393,7 +370,7 @@ __device__ __forceinline__ void team_loop(const JobDev& jb, bool write, uint32_t
                     pick = pos ? static_cast<uint32_t>(L) + 1u : 0u;
                     pick |= __shfl_sync(kFull, neg, L) << 16;
                 } else if (over) {
-                    const int my_e = first_past(wl, w0 + (incl - mine), u);
+                    const int my_e = step::first_past(wl, w0 + (incl - mine), u);
                     const uint32_t q = static_cast<uint32_t>(my_e & 3);
                     // bit 17: no positive weight there, the one-warp layout's site 0
                     pick = __shfl_sync(kFull, (4u * lane + q + 1u) | (((neg >> q) & 1u) << 16) | (my_e < 0 ? 1u << 17 : 0u), L);
@@ -402,7 +379,7 @@ __device__ __forceinline__ void team_loop(const JobDev& jb, bool write, uint32_t
                 if (sel != 0) {
                     const uint32_t q = static_cast<uint32_t>(sel) - 1u;
                     const uint2 es = rb[(q >> 2) & (SL - 1u)];
-                    uint32_t sel_site = site_pick(es.x, es.y, static_cast<int>(q & 3u));
+                    uint32_t sel_site = step::site_pick(es.x, es.y, static_cast<int>(q & 3u));
                     int s_b = (pick & 0x10000u) ? -1 : 1;
                     if (pick >> 17) {
                         W zero;
