@@ -12,7 +12,8 @@
 // overlap pairs share the CTA) and fills its chains' slices of the launch's
 // shared memory with its own run's slice size.  Each item runs exactly the
 // code of the per-class variant with the same lanes, rows and register
-// budget (run_item in sk_step.cuh), so trajectories and records are the same
+// budget (run_item in sk_step.cuh; Gaussian K of 33 to 64 keeps four slots per
+// lane here, the same sums), so trajectories and records are the same
 // as those of whole-warp per-class launches bit for bit.
 #include <cuda_runtime.h>
 #include <stdint.h>
@@ -53,14 +54,14 @@ __global__ void __launch_bounds__(kFusedMaxThreads, 1)
         }
         const uint32_t pc = wi.pad & 0xFFFFFFu;  // the run's shared bytes per chain
         switch (wi.pad >> 24) {                  // fused_variant
-            case 0: step::run_item<int8_t, 0, 1, 32, 0, 8, false>(wi, jb, smem, bars, s_wt, nsteps, pc, phase, dead); break;
-            case 1: step::run_item<int8_t, 0, 2, 32, 0, 8, false>(wi, jb, smem, bars, s_wt, nsteps, pc, phase, dead); break;
-            case 2: step::run_item<int8_t, 1, 1, 32, 0, 8, false>(wi, jb, smem, bars, s_wt, nsteps, pc, phase, dead); break;
-            case 3: step::run_item<int8_t, 1, 1, 32, 0, 8, true>(wi, jb, smem, bars, s_wt, nsteps, pc, phase, dead); break;
-            case 4: step::run_item<float, 0, 1, 32, 0, 8, false>(wi, jb, smem, bars, s_wt, nsteps, pc, phase, dead); break;
-            case 5: step::run_item<float, 0, 2, 32, 0, 8, false>(wi, jb, smem, bars, s_wt, nsteps, pc, phase, dead); break;
-            case 6: step::run_item<float, 1, 1, 32, 0, 8, false>(wi, jb, smem, bars, s_wt, nsteps, pc, phase, dead); break;
-            default: step::run_item<float, 1, 1, 32, 0, 8, true>(wi, jb, smem, bars, s_wt, nsteps, pc, phase, dead); break;
+            case 0: step::run_item<int8_t, 0, 1, 32, 0, 8, false, true>(wi, jb, smem, bars, s_wt, nsteps, pc, phase, dead); break;
+            case 1: step::run_item<int8_t, 0, 2, 32, 0, 8, false, true>(wi, jb, smem, bars, s_wt, nsteps, pc, phase, dead); break;
+            case 2: step::run_item<int8_t, 1, 1, 32, 0, 8, false, true>(wi, jb, smem, bars, s_wt, nsteps, pc, phase, dead); break;
+            case 3: step::run_item<int8_t, 1, 1, 32, 0, 8, true, true>(wi, jb, smem, bars, s_wt, nsteps, pc, phase, dead); break;
+            case 4: step::run_item<float, 0, 1, 32, 0, 8, false, true>(wi, jb, smem, bars, s_wt, nsteps, pc, phase, dead); break;
+            case 5: step::run_item<float, 0, 2, 32, 0, 8, false, true>(wi, jb, smem, bars, s_wt, nsteps, pc, phase, dead); break;
+            case 6: step::run_item<float, 1, 1, 32, 0, 8, false, true>(wi, jb, smem, bars, s_wt, nsteps, pc, phase, dead); break;
+            default: step::run_item<float, 1, 1, 32, 0, 8, true, true>(wi, jb, smem, bars, s_wt, nsteps, pc, phase, dead); break;
         }
         __syncthreads();  // s_job, s_wt and the slices are reused by the next item
     }

@@ -23,7 +23,8 @@
 //       K <= 32 and one block per lane (16- and 32-lane groups), the blocks
 //       of G/SL steps are drawn in one pass (draw_site_batch) and handed out
 //       by shuffles, and whole-warp groups then hold one slot per lane,
-//       d = l + 1 (take_site1): the same draws, hence the same choices.
+//       d = l + 1 (take_site1): the same draws, hence the same choices; with
+//       K <= 64 whole-warp groups hold two slots per lane (take_site2).
 //   a2  the row of J at a = site_1 of the NEXT step is staged by TMA.
 //   a3  candidate energies: centre root dE_d = 2 s_i h_i (i = site_d);
 //       leaf root dE_1 = 2 s_a h_a, dE_d = 2 s_a h_a + 2 s_b h_b - 4 J_ab s_a s_b
@@ -220,6 +221,16 @@ __device__ __forceinline__ void take_site1(uint32_t (&sp)[2], const uint32_t (&b
     const uint32_t w1 = __shfl_sync(g.mask, bat[1], src, G);
     const uint32_t w = (g.gl & 2) ? w1 : w0;
     sp[0] = (w >> (16 * (g.gl & 1))) & 0xFFFFu;
+    sp[1] = 0u;
+}
+// Two slots per lane (slots d = 2 gl + 1, 2 gl + 2, K <= 64 with SL = 16): lane
+// gl takes half gl & 1 of what draw_sites gives lane gl / 2, one word of two sites.
+template <int SL, int G>
+__device__ __forceinline__ void take_site2(uint32_t (&sp)[2], const uint32_t (&bat)[2], uint32_t j, const Grp<G>& g) {
+    const int src = static_cast<int>(j) * SL + (g.gl >> 1);
+    const uint32_t w0 = __shfl_sync(g.mask, bat[0], src, G);
+    const uint32_t w1 = __shfl_sync(g.mask, bat[1], src, G);
+    sp[0] = (g.gl & 1) ? w1 : w0;
     sp[1] = 0u;
 }
 template <int NB>
@@ -593,26 +604,30 @@ __device__ __forceinline__ void chain_loop(const JobDev& jb, bool write, uint32_
     // with no Philox rounds in front of it
     constexpr bool AHEAD2 = STAGED && KEEPW && RULE == 0;
     constexpr bool BATCH = SL > 0;                     // sites in batches of SPB steps
-    constexpr bool SCANSL = BATCH && sizeof(JT) == 1;  // +-J: the scan over SL lanes
+    constexpr bool SCANSL = BATCH && SL <= 8 && sizeof(JT) == 1;  // +-J: the scan over SL lanes
     static_assert(!BATCH || (RULE == 0 && NB == 1 && !STAGED && (SL & (SL - 1)) == 0 && G >= 2 * SL),
                   "site batches: MCMCMC with one block per lane, rows through L1");
     constexpr uint32_t SPB = BATCH ? G / SL : 1;
     // whole-warp groups with site batches hold one slot per lane (slot
     // d = lane + 1, K <= 32), so that a step's candidate work is one slot
     // deep instead of four; their +-J scan covers the first 4 SL lanes
-    constexpr bool SPL1 = BATCH && G == 32;
+    constexpr bool SPL1 = BATCH && G == 32 && SL <= 8;
+    // K of 33 to 64: two slots per lane, where four per lane on 16 lanes left
+    // the other 16 idle through the candidate work and the site draws
+    constexpr bool SPL2 = BATCH && G == 32 && SL == 16;
+    static_assert(!BATCH || SL <= 8 || SPL2, "16 blocks per step: whole-warp groups");
     // the slot weights are kept for the node search also in the throughput
     // variants with two Philox blocks per lane (their register budget holds
     // the 8 weights without spills there; a recomputation costs 4 exponentials
     // and their lookups in the owning lanes of every group) and with one slot
     // per lane (one weight)
-    constexpr bool KEEPXS = KEEPW || NB == 2 || SPL1;
+    constexpr bool KEEPXS = KEEPW || NB == 2 || SPL1 || SPL2;
     // the forms that cost registers or code but fewer dependent instructions
     // (one chain, ns a step: Gaussian N = 512, K = 128 1251 -> 1172, K = 256
     // 1552 -> 1435; the uneven fused batch 3 %): not in the throughput
     // variants, nor in the +-J loop of one slot per lane (533 -> 549 at K = 8)
     constexpr bool LEAN = KEEPW && !(SPL1 && sizeof(JT) == 1);
-    constexpr int NQ = SPL1 ? 1 : 4 * NB;  // slots per lane
+    constexpr int NQ = SPL1 ? 1 : SPL2 ? 2 : 4 * NB;  // slots per lane
     constexpr int SCANL = SPL1 ? (4 * SL < G ? 4 * SL : G) : (SL > 0 ? SL : 1);
     const Grp<G> g;
     // next record point (0: none; a record follows step t when t + 1 == next_rec)
@@ -648,6 +663,8 @@ __device__ __forceinline__ void chain_loop(const JobDev& jb, bool write, uint32_
         draw_site_batch<SL, G>(bat, tb, chain, c3, k0, k1, nblk, N, g);
         if constexpr (SPL1)
             take_site1<SL, G>(site, bat, 0u, g);
+        else if constexpr (SPL2)
+            take_site2<SL, G>(site, bat, 0u, g);
         else
             take_sites<SL, G>(site, bat, 0u, g);
     } else if constexpr (!STAGED && AHEAD && RULE == 0) {
@@ -699,6 +716,8 @@ __device__ __forceinline__ void chain_loop(const JobDev& jb, bool write, uint32_
             }
             if constexpr (SPL1)
                 take_site1<SL, G>(site, bat, j, g);
+            else if constexpr (SPL2)
+                take_site2<SL, G>(site, bat, j, g);
             else
                 take_sites<SL, G>(site, bat, j, g);
         } else if constexpr (!AHEAD && RULE == 0) {
@@ -782,6 +801,8 @@ __device__ __forceinline__ void chain_loop(const JobDev& jb, bool write, uint32_
                     }
                     if constexpr (SPL1)
                         take_site1<SL, G>(nsite, bat, j, g);
+                    else if constexpr (SPL2)
+                        take_site2<SL, G>(nsite, bat, j, g);
                     else
                         take_sites<SL, G>(nsite, bat, j, g);
                 } else if constexpr (!STAGED && AHEAD) {
@@ -795,8 +816,9 @@ __device__ __forceinline__ void chain_loop(const JobDev& jb, bool write, uint32_
                 const H dEa = static_cast<H>(2 * sa) * hf[a];
                 // slot of this lane's entry q
                 auto slot_d = [&](int q) -> uint32_t {
-                    return SPL1 ? static_cast<uint32_t>(g.gl) + 1u
-                                : 4u * G * (q >> 2) + 4u * g.gl + static_cast<uint32_t>(q & 3) + 1u;
+                    return SPL1   ? static_cast<uint32_t>(g.gl) + 1u
+                           : SPL2 ? 2u * static_cast<uint32_t>(g.gl) + static_cast<uint32_t>(q) + 1u
+                                  : 4u * G * (q >> 2) + 4u * g.gl + static_cast<uint32_t>(q & 3) + 1u;
                 };
                 H dE[4 * NB];
                 H mloc = 0;
@@ -853,11 +875,37 @@ __device__ __forceinline__ void chain_loop(const JobDev& jb, bool write, uint32_
                 } else {
                     w0 = dev::pow2(fmaf(-nbl2, m, leaf ? jb.lleaf : jb.lcen));
                 }
+                // two slots per lane, Gaussian: the sums of the four-per-lane form,
+                // taken in the odd lanes (lane 2 v + 1 the four slots of block
+                // v), which the even ones pass their weights and sites to
+                constexpr bool PAIRS = SPL2 && sizeof(JT) == 4;
+                W x4[4] = {W(0), W(0), W(0), W(0)};
+                uint32_t site_even = 0;
+                if constexpr (PAIRS) {
+                    x4[0] = __shfl_up_sync(g.mask, xs[0], 1, G);
+                    x4[1] = __shfl_up_sync(g.mask, xs[1], 1, G);
+                    site_even = __shfl_up_sync(g.mask, site[0], 1, G);
+                    x4[2] = xs[0];
+                    x4[3] = xs[1];
+                    W sum = 0;
+#pragma unroll
+                    for (int e = 0; e < 4; ++e) sum += x4[e];
+                    gsum_[0] = sum;
+                }
                 W incl[NB], tot[NB];
                 W total = w0;
 #pragma unroll
                 for (int q = 0; q < NB; ++q) {
-                    if constexpr (SCANSL) {  // slots in lanes 0 .. SCANL-1 only
+                    if constexpr (PAIRS) {  // over the 16 odd lanes (the even ones' values are not used)
+                        W v = gsum_[0];
+#pragma unroll
+                        for (int o = 2; o < G; o <<= 1) {
+                            const W y = __shfl_up_sync(g.mask, v, o, G);
+                            if (g.gl >= o) v += y;
+                        }
+                        incl[q] = v;
+                        tot[q] = gshfl(g, v, G - 1);
+                    } else if constexpr (SCANSL) {  // slots in lanes 0 .. SCANL-1 only
                         incl[q] = gscan_first<SCANL>(g, gsum_[q]);
                         tot[q] = gshfl(g, incl[q], SCANL - 1);
                     } else {
@@ -897,13 +945,36 @@ __device__ __forceinline__ void chain_loop(const JobDev& jb, bool write, uint32_
                         }
                     }
                 }
+                if constexpr (PAIRS) {
+                    const unsigned over = gballot(g, !found && (g.gl & 1) && base + incl[0] > u);
+                    if (over) {
+                        const int L = __ffs(over) - 1;
+                        const int my_e = first_past(x4, base + (incl[0] - gsum_[0]), u);
+                        const uint32_t my_site =
+                            my_e < 0 ? 0u : (((my_e & 2) ? site[0] : site_even) >> (16 * (my_e & 1))) & 0xFFFFu;
+                        const uint32_t packed = gshfl(g, (my_site << 2) | static_cast<uint32_t>(my_e & 3), L);
+                        sel_site = packed >> 2;
+                        sel_d = 4 * (L >> 1) + static_cast<int>(packed & 3u) + 1;
+                        found = true;
+                    }
+                } else if constexpr (SPL2) {  // +-J: exact sums, two slots per lane in lane order
+                    const unsigned over = gballot(g, !found && base + incl[0] > u);
+                    if (over) {
+                        const int L = __ffs(over) - 1;
+                        const int my_e = base + (incl[0] - gsum_[0]) + xs[0] > u ? 0 : 1;
+                        const uint32_t packed = gshfl(g, (site_of<NB>(site, my_e) << 1) | static_cast<uint32_t>(my_e), L);
+                        sel_site = packed >> 1;
+                        sel_d = 2 * L + static_cast<int>(packed & 1u) + 1;
+                        found = true;
+                    }
+                }
                 // Gaussian weights with several blocks per lane: all blocks'
                 // ballots first (a block's only where no earlier one holds u),
                 // then one search in the block that does, so that the groups of
                 // a warp search together even when their draws fall in
                 // different blocks (for the 64-bit +-J weights the selects cost
                 // more than the second pass they save)
-                constexpr bool ONESEARCH = KEEPXS && !SPL1 && NB > 1 && sizeof(JT) == 4;
+                constexpr bool ONESEARCH = KEEPXS && !SPL1 && !SPL2 && NB > 1 && sizeof(JT) == 4;
                 if constexpr (ONESEARCH) {
                     unsigned ballq[NB];
                     W baseq[NB];
@@ -978,7 +1049,7 @@ __device__ __forceinline__ void chain_loop(const JobDev& jb, bool write, uint32_
                     }
                 }
 #pragma unroll
-                for (int q = 0; q < ((SPL1 || ONESEARCH) ? 0 : NB); ++q) {
+                for (int q = 0; q < ((SPL1 || SPL2 || ONESEARCH) ? 0 : NB); ++q) {
                     const unsigned ball =
                         gballot(g, !found && base + incl[q] > u && (!SCANSL || g.gl < SCANL));
                     if (!found && ball) {
@@ -1097,7 +1168,8 @@ __device__ __forceinline__ void chain_loop(const JobDev& jb, bool write, uint32_
 // operands of a recomputing run, counters).  Warps without a chain meet the
 // CTA's record barriers only.  The job descriptor `jb` (and, +-J, the start of
 // the weight table in `s_wt`) is in shared memory, filled by the caller.
-template <typename JT, int RULE, int NB, int G, int STAGE, int UNROLL, bool RCH>
+// FUSED: one of the loops the fused launch's kernel holds side by side.
+template <typename JT, int RULE, int NB, int G, int STAGE, int UNROLL, bool RCH, bool FUSED = false>
 __device__ __forceinline__ void run_item(const WorkItem& wi, const JobDev& jb, unsigned char* smem, uint64_t* bars,
                                          const unsigned long long* s_wt, uint32_t nsteps, uint32_t per_chain,
                                          uint32_t& phase, bool& dead) {
@@ -1152,6 +1224,9 @@ __device__ __forceinline__ void run_item(const WorkItem& wi, const JobDev& jb, u
             constexpr bool kBatch = RULE == 0 && NB == 1 && STAGE != 1 && (UNROLL >= 8 || G >= 16);
             constexpr int kSL2 = kBatch && G >= 4 ? 2 : 0;
             constexpr int kSL8 = kBatch && G >= 16 ? 8 : 0;
+            // (not the Gaussian one in the fused kernel, where it gains least
+            // and the extra loop costs the others 2 % by spilled registers)
+            constexpr int kSL16 = kBatch && G == 32 && !(FUSED && sizeof(JT) == 4) ? 16 : 0;
             auto loop = [&](auto fast_c, auto sl_c) {
                 chain_loop<JT, RULE, NB, G, STAGE, UNROLL, RCH, decltype(fast_c)::value, decltype(sl_c)::value>(
                     jb, own, chain, cm, partner_off, t0, t1, acc, phase, dead, n_flips, n_rows);
@@ -1165,6 +1240,9 @@ __device__ __forceinline__ void run_item(const WorkItem& wi, const JobDev& jb, u
             } else if (kSL8 && K <= 4u * kSL8) {
                 if (fast) loop(Fast{}, std::integral_constant<int, kSL8>{});
                 else loop(Slow{}, std::integral_constant<int, kSL8>{});
+            } else if (kSL16 && K <= 4u * kSL16) {
+                if (fast) loop(Fast{}, std::integral_constant<int, kSL16>{});
+                else loop(Slow{}, std::integral_constant<int, kSL16>{});
             } else if (fast) {
                 loop(Fast{}, std::integral_constant<int, 0>{});
             } else {

@@ -197,3 +197,41 @@ def test_team_results_are_those_of_one_warp_per_chain(K, rule, p_center, lanes, 
         b.close(); run.close(); inst.close()
     for o in outs[1:]:
         assert all(np.array_equal(x, y) for x, y in zip(outs[0], o))
+
+
+@pytest.mark.parametrize("K", [33, 36, 47, 63, 64])
+@pytest.mark.parametrize("warps", [4, 24, 32])
+def test_two_slots_per_lane(K, warps):
+    # whole-warp chains with K of 33 to 64 hold two slots per lane: +-J against
+    # the oracle (short and long weight tables, traced and not, a non-uniform
+    # root); Gaussian bit for bit against 16 lanes with four slots each
+    need_gpu()
+    N, chains, steps = 77, 2 * warps + 1, 151
+    init = inputs.initial_spins(chains, N, 52)
+
+    def go(J, lanes, scale, trace, p_center):
+        inst = sk.Instance(J, scale=scale)
+        run = sk.Run(inst, chains=chains, K=K, beta=1.1, seed=53, record_every=50, max_records=3, init=init,
+                     trace_chains=chains if trace else 0, trace_steps=steps if trace else 0, p_center=p_center)
+        b = sk.Batch([run], warps_per_cta=warps)
+        b.set_layout(lanes=lanes, staging=2)
+        for n in (1, 50, 100):
+            b.advance(n)
+        E, q, acc = run.observables()
+        out = (run.trace() if trace else None, E, q, acc) + run.state(fields=True)
+        b.close(); run.close(); inst.close()
+        return out
+
+    J = inputs.couplings_pm1(N, 51)
+    for scale, trace, pc in ((1.0, False, 0.0), (1.0, True, 0.3), (0.1, False, 0.0)):
+        g = go(J, 32, scale, trace, pc)
+        o = oracle.run(J, K=K, beta=1.1, seed=53, chains=chains, init=init, steps=steps, record_every=50, trace=True,
+                       scale=scale, p_center=pc)
+        assert np.array_equal(g[1], o["E"]) and np.array_equal(g[3], o["acc"]) and np.array_equal(g[4], o["spins"])
+        if trace:
+            assert np.array_equal(g[0], o["trace"])
+    Jg = inputs.couplings_gauss(N, 54)
+    for pc in (0.0, 0.1):
+        a, b = go(Jg, 32, 1.0, True, pc), go(Jg, 16, 1.0, True, pc)
+        for k in (0, 2, 3, 4, 5, 6):  # (record energies, entry 1, are summed in the order of the lanes)
+            assert np.array_equal(a[k], b[k]), k
