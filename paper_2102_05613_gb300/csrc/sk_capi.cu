@@ -510,30 +510,21 @@ sk_status init_commit(sk_run* r, const int8_t* dinit, bool on_side) {
         SK_CU(cudaEventRecord(in->ev_side, r->stage_st ? r->stage_st : in->side));
         SK_CU(cudaStreamWaitEvent(in->st, in->ev_side, 0));
     }
-    SK_CU(cudaMemsetAsync(r->dstep, 0, sizeof(uint64_t), cs));
-    SK_CU(cudaMemsetAsync(r->derr, 0, sizeof(int), cs));
-    const uint64_t R = r->p.max_records;
-    if (R && r->p.record_every) {
-        SK_CU(cudaMemsetAsync(r->drecE, 0, R * r->chains * sizeof(double), cs));
-        SK_CU(cudaMemsetAsync(r->drecAcc, 0, R * r->chains * sizeof(uint32_t), cs));
-        if (r->chains >= 2) SK_CU(cudaMemsetAsync(r->drecQ, 0, R * (r->chains / 2) * sizeof(double), cs));
-        if (r->drecEnw) SK_CU(cudaMemsetAsync(r->drecEnw, 0, R * r->chains * sizeof(double), cs));
-    }
-    if (r->dtrace)
-        SK_CU(cudaMemsetAsync(r->dtrace, 0xff, static_cast<size_t>(r->p.trace_chains) * r->p.trace_steps * 4, cs));
-    // spins, then the fields h = J s on the tensor cores (e4m3 for +-J:
-    // exact; three bf16 terms of J for Gaussian couplings: fp32 accumulation)
-    SK_CU(sk::launch_init(&r->job, dinit, r->chains, in->N, in->Npad, in->kind, cs, false));
+    // counters, records, statistics and spins in one launch, then the fields
+    // h = J s on the tensor cores (e4m3 for +-J: exact; three bf16 terms of J
+    // for Gaussian couplings: fp32 accumulation)
+    if (sk_status s = ensure_recompute(r, cs); s != SK_OK) return s;
+    sk::StartJob sj{};
+    sj.job = r->job;
+    sj.init = dinit;
+    sj.dstats = r->dstats;
+    sj.ddE = r->ddE;
+    sj.s_op = r->dSop;
+    SK_CU(sk::launch_start_one(sj, cs));
     if (dinit == r->dstage && dinit) SK_CU(cudaEventRecord(r->ev_sfree, cs));
-    {
-        sk_status s = ensure_recompute(r, cs);
-        if (s != SK_OK) return s;
-        SK_CU(sk::launch_recompute(in->kind, r->ds, r->dh, nullptr, r->dSop, in->dJop, r->ddE, r->dstats,
-                                   r->derr, r->chains, in->Npad, 3, 3, in->scale, cs));
-        r->sop_valid = true;  // the conversion of the start spins
-    }
-    SK_CU(cudaMemsetAsync(r->dstats, 0, 6 * sizeof(unsigned long long), cs));
-    SK_CU(cudaMemsetAsync(r->ddE, 0, static_cast<size_t>(r->chains) * sizeof(double), cs));
+    SK_CU(sk::launch_recompute(in->kind, r->ds, r->dh, nullptr, r->dSop, in->dJop, r->ddE, r->dstats, r->derr, r->chains,
+                               in->Npad, 3, 3, in->scale, cs, 0, true));
+    r->sop_valid = true;
     if (on_side) {
         SK_CU(cudaEventRecord(in->ev_side, in->side));
         SK_CU(cudaStreamWaitEvent(in->st, in->ev_side, 0));

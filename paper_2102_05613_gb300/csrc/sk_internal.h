@@ -123,6 +123,7 @@ struct StartJob {
     void* s_op;                  // or null: the spins also written as tensor-core operands
                                  // (e4m3 for +-J, bf16 for Gaussian couplings)
 };
+cudaError_t launch_start_one(const StartJob& job, cudaStream_t st);
 cudaError_t launch_start_batch(const StartJob* jobs_dev, uint32_t n, uint64_t max_words, cudaStream_t st);
 // Device checks of host-supplied inputs: *flag receives the smallest
 // (position << 2 | code) of a violation, all ones when there is none
