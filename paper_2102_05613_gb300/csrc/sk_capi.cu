@@ -303,7 +303,7 @@ struct sk_run {
     cudaStream_t stage_st = nullptr;  // where the last spins stage was made (input_stream() or side)
     cudaEvent_t ev_sfree = nullptr;  // st: the start kernel has read dstage
     unsigned long long* dflag = nullptr;  // result word of the start-spin check
-    unsigned long long* hflag = nullptr;  // its pinned host copy
+    unsigned long long* hflag = nullptr;  // pinned: its host copy, and the error word's
     uint32_t* dacc = nullptr;
     unsigned long long* dwork = nullptr;
     double* drecE = nullptr;
@@ -431,10 +431,15 @@ sk_status upload_couplings(sk_instance* in, const void* J, uint32_t mem, bool fr
     return couplings_commit(in, fresh);
 }
 
+// Waits for the run's stream and reports an error its kernels left: the copy
+// of the error word (into pinned memory) is queued behind the work and one
+// wait covers both.  (Polling the stream with 50 us sleeps and then copying
+// the word into pageable memory cost a short run 50 to 100 us.)
 sk_status check_run_error(sk_run* r) {
-    int h = 0;
-    SK_CU(cudaMemcpyAsync(&h, r->derr, sizeof(int), cudaMemcpyDeviceToHost, r->inst->st));
+    int* herr = reinterpret_cast<int*>(r->hflag + 1);
+    SK_CU(cudaMemcpyAsync(herr, r->derr, sizeof(int), cudaMemcpyDeviceToHost, r->inst->st));
     SK_CU(cudaStreamSynchronize(r->inst->st));
+    const int h = *herr;
     if (h == sk::kDevTimeout) return fail(SK_ERR_TIMEOUT, "a bounded device wait expired in the step kernel");
     if (h == sk::kDevBounds) return fail(SK_ERR_DEVICE, "a kernel reported an out-of-range index");
     return SK_OK;
@@ -852,7 +857,7 @@ sk_status mcmcmc_create(sk_instance* in, const sk_run_params* p, sk_run** out) {
     if (s == SK_OK && cudaEventCreateWithFlags(&r->ev_sfree, cudaEventDisableTiming) != cudaSuccess)
         s = fail(SK_ERR_CUDA, "event creation failed");
     if (s == SK_OK) s = dalloc(&r->dflag, sizeof(unsigned long long));
-    if (s == SK_OK && cudaHostAlloc(reinterpret_cast<void**>(&r->hflag), sizeof(unsigned long long),
+    if (s == SK_OK && cudaHostAlloc(reinterpret_cast<void**>(&r->hflag), 2 * sizeof(unsigned long long),
                                     cudaHostAllocDefault) != cudaSuccess)
         s = fail(SK_ERR_OOM, "pinned host allocation failed");
     if (s == SK_OK && in->kind == SK_J_PM1) {
@@ -1076,11 +1081,11 @@ sk_status mcmcmc_observables_many(sk_run* const* runs, uint32_t n, uint64_t firs
 sk_status mcmcmc_wait(sk_run* r, uint64_t timeout_ns) {
     if (!r) return fail(SK_ERR_INVALID_ARG, "run is NULL");
     const auto t0 = std::chrono::steady_clock::now();
-    for (;;) {
+    while (timeout_ns) {  // (no limit: check_run_error waits)
         cudaError_t e = cudaStreamQuery(r->inst->st);
         if (e == cudaSuccess) break;
         if (e != cudaErrorNotReady) return fail(SK_ERR_CUDA, "stream: %s", cudaGetErrorString(e));
-        if (timeout_ns) {
+        {
             const auto ns = std::chrono::duration_cast<std::chrono::nanoseconds>(
                                 std::chrono::steady_clock::now() - t0).count();
             if (static_cast<uint64_t>(ns) >= timeout_ns)
@@ -1139,7 +1144,7 @@ sk_status mcmcmc_state(sk_run* r, int8_t* spins, void* fields, uint64_t* step, u
     if (fields)
         SK_CU(cudaMemcpy2DAsync(fields, in->N * 4, r->dh, in->Npad * 4, in->N * 4, r->chains, cudaMemcpyDefault, st));
     uint64_t ds = 0;
-    SK_CU(cudaMemcpyAsync(&ds, r->dstep, 8, cudaMemcpyDeviceToHost, st));
+    if (step) SK_CU(cudaMemcpyAsync(&ds, r->dstep, 8, cudaMemcpyDeviceToHost, st));
     SK_CU(cudaStreamSynchronize(st));
     if (step) *step = ds;
     return SK_OK;
