@@ -49,6 +49,19 @@ constexpr uint32_t EW = 8;                                 // epilogue warps: 2 
 constexpr uint32_t SMEM_BYTES = NS * STAGE_BYTES + 1024;  // + 1 KB alignment slack
 constexpr uint32_t TMEM_COLS = 512;                        // two 256-column accumulators
 constexpr uint32_t WS_THREADS = 64 + 32 * EW;              // producer, MMA, epilogue warps
+// MT row blocks of 128 per tile.  MT = 1: two accumulators take tiles in turn.
+// MT = 2: a tile is 256 rows, each B tile in shared memory serves two MMAs, one
+// per accumulator: 64 KB instead of 96 KB from L2 for the same products, where
+// the main loop is bound by what an SM takes in from L2 (~64 B per clock).  Its
+// epilogue does not overlap the next tile's main loop, so it is the choice
+// for long sums and many rows (bf16, tall_tiles).  Stages: 192 KB either way.
+template <int MT>
+struct Tile {
+    static constexpr uint32_t kStages = MT == 1 ? NS : 3u;
+    static constexpr uint32_t kStageBytes = MT * TILE_A + TILE_B;
+    static constexpr uint32_t kRows = MT * BM;
+};
+static_assert(Tile<2>::kStages * Tile<2>::kStageBytes == NS * STAGE_BYTES, "same shared memory");
 constexpr long long kBudget = 4000000000ll;  // ~2 s of clock cycles per wait
 
 __device__ __forceinline__ uint32_t saddr(const void* p) {
@@ -269,7 +282,7 @@ __device__ __forceinline__ void epilogue_rows(uint32_t taddr, const Args& args, 
             atomicMax(&args.stats[0], static_cast<unsigned long long>(__double_as_longlong(dmax)));
             if (mw) atomicAdd(&args.stats[1], static_cast<unsigned long long>(mw));
         }
-        if (args.cnt) {
+        if (args.cnt && row0 < args.chains) {
             // the energy drift of these 32 chains is complete once the epilogue
             // warps of all their tiles (two column halves each) have added to
             // it: the last of them takes |scale/2 dE| of each chain into the
@@ -343,7 +356,7 @@ __device__ __forceinline__ void energy_rows(uint32_t taddr, const Args& args, ui
 // slice of one output tile, whose K range starts at the tile's own columns
 // (what lies before them is zero), and the tasks with the longest range come
 // first, so that the last round of the persistent CTAs is a short one.
-template <bool F8, int KIND>
+template <bool F8, int KIND, int MT = 1>
 __global__ void __launch_bounds__(WS_THREADS, 1)
     recompute_ws_kernel(const __grid_constant__ CUtensorMap tA, const __grid_constant__ CUtensorMap tB0,
                         const __grid_constant__ CUtensorMap tB1, const __grid_constant__ CUtensorMap tB2,
@@ -351,8 +364,10 @@ __global__ void __launch_bounds__(WS_THREADS, 1)
                         uint32_t ntasks, uint32_t tiles_n) {
     constexpr bool BATCH = KIND == 1;
     constexpr bool ENERGY = KIND == 2;
+    constexpr uint32_t kNS = Tile<MT>::kStages, kSB = Tile<MT>::kStageBytes;
+    static_assert(MT == 1 || (!F8 && !ENERGY), "256-row tiles: bf16 recompute");
     extern __shared__ __align__(1024) unsigned char smem_raw[];
-    __shared__ __align__(8) uint64_t full[NS], empty[NS], tfull[2], tempty[2], drain;
+    __shared__ __align__(8) uint64_t full[kNS], empty[kNS], tfull[2], tempty[2], drain;
     __shared__ uint32_t tmem_holder;
     __shared__ int dead;
     // 128-byte-swizzled tiles must start on a 1024-byte boundary of shared memory
@@ -363,7 +378,7 @@ __global__ void __launch_bounds__(WS_THREADS, 1)
     volatile int* vdead = &dead;
 
     if (threadIdx.x == 0) {
-        for (uint32_t i = 0; i < NS; ++i) {
+        for (uint32_t i = 0; i < kNS; ++i) {
             asm volatile("mbarrier.init.shared::cta.b64 [%0], 1;" ::"r"(saddr(&full[i])) : "memory");
             asm volatile("mbarrier.init.shared::cta.b64 [%0], 1;" ::"r"(saddr(&empty[i])) : "memory");
         }
@@ -414,7 +429,7 @@ __global__ void __launch_bounds__(WS_THREADS, 1)
                 m0 = (t % tiles_m) * BM;
                 n0 = a->b_row0 + (t / (tiles_m * slices)) * BN;
             } else {
-                m0 = (t / tiles_n) * BM;
+                m0 = (t / tiles_n) * (MT * BM);
                 n0 = (t % tiles_n) * BN;
             }
         }
@@ -439,9 +454,9 @@ __global__ void __launch_bounds__(WS_THREADS, 1)
                 const uint32_t total = ENERGY ? a->kblocks - kb0 : a->terms * a->kblocks;
                 const uint32_t brow = ENERGY ? slice_of(t) * a->b_rows + n0 - a->b_row0 : n0;
                 for (uint32_t i = 0; i < total; ++i, ++g) {
-                    const uint32_t st = g % NS;
-                    if (a->compute_only && g >= NS) break;  // the probe fills the ring once
-                    if (g >= NS && !wait_bounded(saddr(&empty[st]), ((g / NS) - 1u) & 1u)) {
+                    const uint32_t st = g % kNS;
+                    if (a->compute_only && g >= kNS) break;  // the probe fills the ring once
+                    if (g >= kNS && !wait_bounded(saddr(&empty[st]), ((g / kNS) - 1u) & 1u)) {
                         atomicExch(a->err, kDevTimeout);
                         *vdead = 1;
                     }
@@ -451,20 +466,23 @@ __global__ void __launch_bounds__(WS_THREADS, 1)
                         continue;
                     }
                     const uint32_t term = ENERGY ? 0u : i / a->kblocks, kb = ENERGY ? kb0 + i : i % a->kblocks;
-                    unsigned char* sa = smem + st * STAGE_BYTES;
+                    unsigned char* sa = smem + st * kSB;
                     asm volatile("mbarrier.arrive.expect_tx.shared::cta.b64 _, [%0], %1;" ::"r"(saddr(&full[st])),
-                                 "r"(STAGE_BYTES)
+                                 "r"(kSB)
                                  : "memory");
-                    tma_2d(saddr(sa), A, static_cast<int>(kb * kElems), static_cast<int>(m0), saddr(&full[st]));
-                    tma_2d(saddr(sa + TILE_A), B[term], static_cast<int>(kb * kElems), static_cast<int>(brow),
+#pragma unroll
+                    for (int mt = 0; mt < MT; ++mt)
+                        tma_2d(saddr(sa + mt * TILE_A), A, static_cast<int>(kb * kElems),
+                               static_cast<int>(m0 + mt * BM), saddr(&full[st]));
+                    tma_2d(saddr(sa + MT * TILE_A), B[term], static_cast<int>(kb * kElems), static_cast<int>(brow),
                            saddr(&full[st]));
                 }
             }
-            // the copies of the last NS stages issued have landed before the
+            // the copies of the last stages issued have landed before the
             // CTA may leave (at once after a normal run, where the MMA warp
             // consumed them; bounded after an expired wait)
-            for (uint32_t q = g > NS ? g - NS : 0u; q < g; ++q)
-                if (q != withheld) wait_bounded(saddr(&full[q % NS]), (q / NS) & 1u);
+            for (uint32_t q = g > kNS ? g - kNS : 0u; q < g; ++q)
+                if (q != withheld) wait_bounded(saddr(&full[q % kNS]), (q / kNS) & 1u);
         }
     } else if (warp == 1) {
         if (lane == 0) {  // MMA issuer: 4 MMAs of K = 32 bytes per stage into accumulator j % 2
@@ -475,8 +493,9 @@ __global__ void __launch_bounds__(WS_THREADS, 1)
                 const Args* a;
                 uint32_t m0, n0;
                 task(t, A, B, a, m0, n0);
-                const uint32_t b = j & 1u;
-                if (j >= 2 && !wait_bounded(saddr(&tempty[b]), ((j >> 1) - 1u) & 1u)) {  // epilogue done with it
+                // MT = 1: accumulator j % 2; MT = 2: both, one tile at a time
+                const uint32_t b = MT == 1 ? j & 1u : 0u, use = MT == 1 ? j >> 1 : j;
+                if (use >= 1 && !wait_bounded(saddr(&tempty[b]), (use - 1u) & 1u)) {  // epilogue done with it
                     atomicExch(a->err, kDevTimeout);
                     *vdead = 1;
                     break;
@@ -485,19 +504,22 @@ __global__ void __launch_bounds__(WS_THREADS, 1)
                 const uint32_t acc = tmem + 256u * b;
                 const uint32_t total = ENERGY ? a->kblocks - n0 / kElems : a->terms * a->kblocks;
                 for (uint32_t i = 0; i < total; ++i, ++g) {
-                    const uint32_t st = g % NS;
+                    const uint32_t st = g % kNS;
                     // (the probe waits for each stage once, then reuses it)
-                    if ((!a->compute_only || g < NS) && !wait_bounded(saddr(&full[st]), (g / NS) & 1u)) {
+                    if ((!a->compute_only || g < kNS) && !wait_bounded(saddr(&full[st]), (g / kNS) & 1u)) {
                         atomicExch(a->err, kDevTimeout);
                         *vdead = 1;
                     }
                     if (*vdead) break;
                     asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
-                    const uint32_t sa = saddr(smem + st * STAGE_BYTES);
-                    const uint32_t sb = sa + TILE_A;
+                    const uint32_t sa = saddr(smem + st * kSB);
+                    const uint32_t sb = sa + MT * TILE_A;
 #pragma unroll
                     for (uint32_t kk = 0; kk < 4; ++kk)
-                        mma<F8>(acc, sw128_desc(sa + 32 * kk), sw128_desc(sb + 32 * kk), idesc, (i | kk) != 0u);
+#pragma unroll
+                        for (uint32_t mt = 0; mt < MT; ++mt)
+                            mma<F8>(acc + 256u * mt, sw128_desc(sa + mt * TILE_A + 32 * kk), sw128_desc(sb + 32 * kk),
+                                    idesc, (i | kk) != 0u);
                     if (!a->compute_only) mma_commit(saddr(&empty[st]));
                 }
                 mma_commit(saddr(&tfull[b]));  // completes when the tile's MMAs have
@@ -521,14 +543,14 @@ __global__ void __launch_bounds__(WS_THREADS, 1)
             const Args* a;
             uint32_t m0, n0;
             task(t, A, B, a, m0, n0);
-            const uint32_t b = j & 1u;
+            const uint32_t b = MT == 1 ? j & 1u : 0u, use = MT == 1 ? j >> 1 : j;
             // the first column block's fields and spins do not depend on the
             // accumulator: their loads go out before the wait for it
             RowBlock first;
             if (!ENERGY && !a->compute_only)
                 load_row_block(first, *a, m0 + qd * 32u + lane, n0 + half * (BN / 2), m0 + qd * 32u + lane < a->chains);
             // every lane waits; the outcome is made warp-uniform
-            const bool ok = __all_sync(0xffffffffu, !*vdead && wait_bounded(saddr(&tfull[b]), (j >> 1) & 1u));
+            const bool ok = __all_sync(0xffffffffu, !*vdead && wait_bounded(saddr(&tfull[b]), use & 1u));
             if (!ok && lane == 0) {
                 atomicExch(a->err, kDevTimeout);
                 *vdead = 1;
@@ -538,9 +560,15 @@ __global__ void __launch_bounds__(WS_THREADS, 1)
             if constexpr (ENERGY)
                 energy_rows(tmem + ((qd * 32u) << 16) + 256u * b, *a, m0 + qd * 32u, n0, half * (BN / 2),
                             slice_of(t), ok && live);
-            else if (!a->compute_only)
+            else if (!a->compute_only) {
                 epilogue_rows(tmem + ((qd * 32u) << 16) + 256u * b, *a, m0 + qd * 32u, n0, half * (BN / 2),
                               ok && live, first);
+                if constexpr (MT == 2) {
+                    const uint32_t row0 = m0 + BM + qd * 32u;
+                    load_row_block(first, *a, row0 + lane, n0 + half * (BN / 2), row0 + lane < a->chains);
+                    epilogue_rows(tmem + ((qd * 32u) << 16) + 256u, *a, row0, n0, half * (BN / 2), ok && live, first);
+                }
+            }
             asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
             __syncwarp();
             if (lane == 0) mbar_arrive(saddr(&tempty[b]));
@@ -710,6 +738,38 @@ cudaError_t recompute_prepare_j(const void* J, uint32_t kind, uint32_t npad, voi
 }
 
 namespace {
+// Whether 256-row tiles (bf16) finish first: rounds of the persistent CTAs times
+// the main loop (us a 128-byte K block: 0.47 on 128-row tiles, 0.57 on 256-row
+// ones) and the epilogue of a row block (8.5 us where it reads the old fields
+// and spins, 6 where it only writes), which overlaps the main loop on 128-row
+// tiles only.  Resync of three terms, 128 / 256 rows: N = 2048 x 8192 chains
+// 191 / 135 us, 1024 x 16384 123 / 82, 2048 x 4096 101 / 68; the check of
+// 512 x 65536, 108 / 129, keeps the 128.  FP8 tiles stay at 128: 2048 x 8192
+// took 50 / 60 us, the best other size 42 / 40.
+bool tall_tiles(uint64_t tiles128, uint64_t tiles256, uint32_t kblocks, bool reads) {
+    const uint64_t sms = static_cast<uint64_t>(sm_count());
+    const double e = reads ? 8.5 : 6.0;
+    const double t1 = static_cast<double>((tiles128 + sms - 1) / sms) * std::max(0.47 * kblocks, e);
+    const double t2 = static_cast<double>((tiles256 + sms - 1) / sms) * (0.57 * kblocks + 2.0 * e);
+    return t2 < t1;
+}
+
+// The dynamic shared-memory attribute of a recompute kernel variant, set once
+// per device and variant.
+template <typename F>
+cudaError_t smem_attribute(F kernel, int variant) {
+    static std::mutex mu;
+    static std::set<std::pair<int, int>> done;
+    int dev = 0;
+    cudaError_t e = cudaGetDevice(&dev);
+    if (e != cudaSuccess) return e;
+    std::lock_guard<std::mutex> lk(mu);
+    if (done.count({dev, variant})) return cudaSuccess;
+    e = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, SMEM_BYTES);
+    if (e == cudaSuccess) done.insert({dev, variant});
+    return e;
+}
+
 // The coupling operands of several instances of one kind in one launch
 // (blockIdx.y = instance): the conversions of pm1_to_e4m3 / gauss_to_bf16x3.
 __global__ void prepare_j_batch(const PrepareJ* __restrict__ jobs, uint32_t pm1) {
@@ -757,6 +817,7 @@ cudaError_t launch_set_fields_batch(uint32_t kind, const RecomputeSet* sets, uin
     std::vector<BatchJob> jobs(n);
     std::vector<BatchTask> tasks;
     size_t maxn = 0;
+    uint64_t nt1 = 0, nt2 = 0, kb = 0;  // tiles of either height, K blocks of all sets
     for (uint32_t i = 0; i < n; ++i) {
         const RecomputeSet& q = sets[i];
         seg[i] = SegSpins{q.s, q.s_op, static_cast<size_t>(q.chains) * q.npad};
@@ -779,9 +840,15 @@ cudaError_t launch_set_fields_batch(uint32_t kind, const RecomputeSet* sets, uin
         b.args.mode = 3;
         b.args.pm1 = bf ? 0u : 1u;
         b.args.fault = 0u;
-        for (uint32_t m0 = 0; m0 < q.chains; m0 += BM)
-            for (uint32_t n0 = 0; n0 < q.npad; n0 += BN) tasks.push_back(BatchTask{i, m0, n0, 0});
+        const uint64_t tn = (q.npad + BN - 1) / BN;
+        nt1 += (q.chains + BM - 1) / BM * tn;
+        nt2 += (q.chains + 2 * BM - 1) / (2 * BM) * tn;
+        kb += b.args.terms * b.args.kblocks;
     }
+    const bool tall = bf && tall_tiles(nt1, nt2, static_cast<uint32_t>(kb / n), false);
+    for (uint32_t i = 0; i < n; ++i)
+        for (uint32_t m0 = 0; m0 < sets[i].chains; m0 += tall ? 2 * BM : BM)
+            for (uint32_t n0 = 0; n0 < sets[i].npad; n0 += BN) tasks.push_back(BatchTask{i, m0, n0, 0});
     SegSpins* dseg = nullptr;
     BatchJob* djobs = nullptr;
     BatchTask* dtasks = nullptr;
@@ -804,19 +871,14 @@ cudaError_t launch_set_fields_batch(uint32_t kind, const RecomputeSet* sets, uin
         std::memset(&a0, 0, sizeof a0);
         const uint32_t nt = static_cast<uint32_t>(tasks.size());
         const uint32_t grid = std::max<uint32_t>(1u, std::min<uint32_t>(nt, static_cast<uint32_t>(sm_count())));
-        if (bf) {
-            e = cudaFuncSetAttribute(recompute_ws_kernel<false, 1>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                     SMEM_BYTES);
+        auto go = [&](auto kernel, int variant) {
+            e = smem_attribute(kernel, variant);
             if (e == cudaSuccess)
-                recompute_ws_kernel<false, 1><<<grid, WS_THREADS, SMEM_BYTES, st>>>(none, none, none, none, a0,
-                                                                                      djobs, dtasks, nt, 0u);
-        } else {
-            e = cudaFuncSetAttribute(recompute_ws_kernel<true, 1>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                     SMEM_BYTES);
-            if (e == cudaSuccess)
-                recompute_ws_kernel<true, 1><<<grid, WS_THREADS, SMEM_BYTES, st>>>(none, none, none, none, a0,
-                                                                                     djobs, dtasks, nt, 0u);
-        }
+                kernel<<<grid, WS_THREADS, SMEM_BYTES, st>>>(none, none, none, none, a0, djobs, dtasks, nt, 0u);
+        };
+        if (tall) go(recompute_ws_kernel<false, 1, 2>, 5);
+        else if (bf) go(recompute_ws_kernel<false, 1>, 6);
+        else go(recompute_ws_kernel<true, 1>, 7);
         if (e == cudaSuccess) e = cudaGetLastError();
     }
     cudaFreeAsync(dseg, st);
@@ -826,22 +888,6 @@ cudaError_t launch_set_fields_batch(uint32_t kind, const RecomputeSet* sets, uin
 }
 
 namespace {
-// The dynamic shared-memory attribute of a recompute kernel variant, set once
-// per device and variant.
-template <typename F>
-cudaError_t smem_attribute(F kernel, int variant) {
-    static std::mutex mu;
-    static std::set<std::pair<int, int>> done;
-    int dev = 0;
-    cudaError_t e = cudaGetDevice(&dev);
-    if (e != cudaSuccess) return e;
-    std::lock_guard<std::mutex> lk(mu);
-    if (done.count({dev, variant})) return cudaSuccess;
-    e = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, SMEM_BYTES);
-    if (e == cudaSuccess) done.insert({dev, variant});
-    return e;
-}
-
 // Operand tensor maps by (spin operand, coupling operand, type, shape): a map
 // holds only addresses and shapes, so one encoded for the same buffers and
 // shape is valid again; a few recent entries are kept.
@@ -915,10 +961,16 @@ cudaError_t launch_recompute(uint32_t kind, const int8_t* s, void* h, float* out
     a.fault = fault;
     a.compute_only = 0;
     const uint32_t tiles_n = (npad + BN - 1) / BN;
-    const uint32_t nt = ((chains + BM - 1) / BM) * tiles_n;
-    if (nt == 0) return cudaSuccess;
+    const uint32_t nt1 = ((chains + BM - 1) / BM) * tiles_n, nt2 = ((chains + 2 * BM - 1) / (2 * BM)) * tiles_n;
+    if (nt1 == 0) return cudaSuccess;
+    const bool tall = bf && tall_tiles(nt1, nt2, terms * a.kblocks, mode < 2);
+    const uint32_t nt = tall ? nt2 : nt1;
     const uint32_t grid = std::min<uint32_t>(nt, static_cast<uint32_t>(sm_count()));
-    if (bf) {
+    if (tall) {
+        if ((e = smem_attribute(recompute_ws_kernel<false, 0, 2>, 4)) != cudaSuccess) return e;
+        recompute_ws_kernel<false, 0, 2><<<grid, WS_THREADS, SMEM_BYTES, st>>>(tA, tB[0], tB[1], tB[2], a, nullptr,
+                                                                              nullptr, nt, tiles_n);
+    } else if (bf) {
         if ((e = smem_attribute(recompute_ws_kernel<false, 0>, 0)) != cudaSuccess) return e;
         recompute_ws_kernel<false, 0><<<grid, WS_THREADS, SMEM_BYTES, st>>>(tA, tB[0], tB[1], tB[2], a, nullptr,
                                                                                nullptr, nt, tiles_n);

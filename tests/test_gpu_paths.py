@@ -235,3 +235,37 @@ def test_two_slots_per_lane(K, warps):
         a, b = go(Jg, 32, 1.0, True, pc), go(Jg, 16, 1.0, True, pc)
         for k in (0, 2, 3, 4, 5, 6):  # (record energies, entry 1, are summed in the order of the lanes)
             assert np.array_equal(a[k], b[k]), k
+
+
+@pytest.mark.parametrize("N,chains", [(1024, 16301), (2000, 4100)])
+def test_recompute_on_256_row_tiles(N, chains):
+    # enough rows and terms for the 256-row tiles: last tiles with 173 rows and
+    # with 4 (no row in the second half), ragged columns; start fields, drift
+    # figures, both forms of the resync
+    torch = need_gpu()
+    J = torch.from_numpy(inputs.couplings(N, sk.SK_J_GAUSS, 61)).cuda()
+    g = torch.Generator(device="cuda").manual_seed(62)
+    S = (2 * torch.randint(0, 2, (chains, N), generator=g, device="cuda", dtype=torch.int8) - 1).contiguous()
+    inst = sk.Instance(J)
+    run = sk.Run(inst, chains=chains, K=4, beta=1.0, seed=3, init=S)
+
+    def state():
+        s = torch.empty_like(S)
+        h = torch.empty((chains, N), dtype=torch.float32, device="cuda")
+        assert sk.lib().mcmcmc_state(run.handle, C.c_void_p(s.data_ptr()), C.c_void_p(h.data_ptr()), None,
+                                     sk.SK_MEM_DEVICE) == sk.SK_OK
+        return s, h
+    # the tensor core's FP32 accumulator rounds once per MMA step of 16 products
+    tol = max(3e-5, 3 * N / 16 * 2.0 ** -23 * 4)
+    s, h = state()
+    assert torch.equal(s, S) and (h.double() - S.double() @ J.double()).abs().max().item() <= tol
+    run.advance(20)
+    exact = state()[0].double() @ J.double()
+    st, _ = run.recompute(sk.SK_RECOMPUTE_CHECK)
+    assert st["max_field_drift"] <= 2 * tol + 1e-4
+    run.recompute(sk.SK_RECOMPUTE_RESYNC, sync=False)  # enqueued only: sets the fields
+    h1 = state()[1].clone()
+    st, _ = run.recompute(sk.SK_RECOMPUTE_RESYNC)      # with figures: they are the same fields
+    h2 = state()[1]
+    assert torch.equal(h1, h2) and st["max_field_drift"] == 0.0 and (h2.double() - exact).abs().max().item() <= tol
+    run.close(); inst.close()
