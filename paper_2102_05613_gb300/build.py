@@ -21,7 +21,7 @@ SOURCES = ["sk_kernels.cu", "sk_capi.cu", "sk_noalloc.cu", "sk_recompute.cu", "s
            "sk_cluster.cu", "sk_cluster_pm1.cu", "sk_cluster_gauss.cu", "sk_fused.cu",
            "sk_team.cu", "sk_team_pm1.cu", "sk_team_gauss.cu"] + [
     f"sk_step_{c}_{r}_{s}.cu" for c in ("pm1", "gauss") for r in ("mcmcmc", "metropolis")
-    for s in ("staged", "direct", "direct_nw")]
+    for s in ("staged", "direct", "direct_nw")] + ["sk_step_gauss_mcmcmc_direct_sum32.cu"]
 ARCH = ["-gencode", "arch=compute_103a,code=sm_103a"]
 
 

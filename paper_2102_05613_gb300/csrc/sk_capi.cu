@@ -1416,6 +1416,93 @@ uint32_t default_team(const sk_batch* b, const std::vector<uint32_t>& idx, int s
     return 0;
 }
 
+// Lanes per chain and warps per CTA of a class of many chains (more than 32 per
+// SM) that nothing forces or has tuned; G = 0: the whole-warp default.
+//
+// Fewer lanes per chain leave fewer of them idle in the scan, the node search
+// and the draws; where the chains' rows crowd each other out of L1 (N), or a
+// lane's table lookups and exponentials do not spread over enough lanes (long
+// tables, K <= 32 Gaussian), whole warps are faster.  us a step, 32 lanes with
+// 32 / 24 warps a CTA against the fewer lanes; 65,536 chains (N = 768, 1024: 32,768):
+//   Gaussian, 16 lanes, 24 warps: N = 512 K = 64 33.7 / 32.1, 27.9; K = 128 40.4 /
+//     40.8, 34.7; N = 640 K = 128 35.9 / 34.9, 30.2; N = 768 23.2 / 22.0, 26.8
+//   +-J, weight table in shared memory: K = 32, 8 lanes, 16 warps: N = 128 15.3 /
+//     15.2, 10.6; N = 256 15.5 / 15.5, 11.5; N = 512 17.1 / 17.7, 16.8 (K = 8 the
+//     other way); K = 64, 16 lanes, 32 warps: N = 512 20.6 / 20.8, 18.5, N = 768
+//     11.6 / 12.0, 14.7; K = 128, 16 lanes, 24 warps: 30.2 / 29.6, 27.9 and 16.4 / 16.1, 17.0
+//   +-J, longer table: K = 32 N = 256 23.5 / 24.3, 19.9, N = 512 28.9 / 30.3, 28.9;
+//     K = 64 N = 256 29.3 / 28.9, 27.7, N = 512 34.9 / 34.0, 36.4; K = 128 N = 512
+//     53.3 / 52.2, 44.8, N = 768 29.8 / 29.0, 26.9, N = 1024 33.3 / 31.9, 32.4
+//   Metropolis, 16 lanes, 32 warps: Gaussian N = 256 5.4 / 5.6, 4.6, N = 512 7.4 /
+//     7.6, 7.6; +-J short N = 512 5.0 / 5.2, 4.2, N = 768 3.1 / 3.3, 4.0; longer
+//     N = 256 6.2 / 6.2, 4.7, N = 512 7.9 / 8.2, 8.6
+// Whole warps: 24 a CTA (80 registers, no spills) take 2 to 10 % less than 32
+// over many rounds where the weights' search is long (K > 64, K > 32 other than
+// short tables; K = 256 47.8 / 45.2, Gaussian N = 768 K = 64 21.3 / 20.1), more
+// elsewhere.  A few rounds decide by the cost: CTA rounds times a round's
+// time, in whole-warp chains' worth of issue (12,288 Gaussian chains N = 512,
+// K = 128: three rounds of 28 warps 8.5 ms a 1000 steps, two of 16 lanes 7.6).
+struct ManyChains {
+    uint32_t G = 0, W = 0;
+};
+ManyChains many_chains_layout(const sk_batch* b, const std::vector<uint32_t>& idx, uint32_t per_chain, int sms) {
+    const sk_run* r0 = b->runs[idx[0]];
+    const bool pm1 = r0->inst->kind == SK_J_PM1, metropolis = r0->p.rule == SK_RULE_METROPOLIS;
+    uint64_t total = 0;
+    uint32_t K = 1, npad = 0;
+    bool short_tables = pm1;
+    for (uint32_t i : idx) {
+        const sk_run* r = b->runs[i];
+        total += r->chains;
+        K = std::max(K, r->p.K);
+        npad = std::max(npad, r->inst->Npad);
+        short_tables = short_tables && r->wlen <= 64u;
+    }
+    ManyChains best;
+    if (total <= 32u * static_cast<uint64_t>(sms)) return best;
+    auto rounds = [&](uint32_t chains_per_cta) -> double {
+        uint64_t items = 0;
+        for (uint32_t i : idx) items += (b->runs[i]->chains + chains_per_cta - 1) / chains_per_cta;
+        return static_cast<double>((items + sms - 1) / sms);
+    };
+    // a round's fixed part, in chains: long Metropolis and short MCMCMC steps
+    // wait more than they issue
+    const double fixed = metropolis ? 24.0 : K <= 32u ? 12.0 : 2.4;
+    double cost = 1e300;
+    const uint32_t fit32 = std::min(32u, fit_warps(per_chain, 32));
+    if (fit32 < 18) return best;
+    const bool few = rounds(std::min(24u, fit32)) <= 4.0;
+    for (uint32_t W = fit32; W >= 18; W -= 2) {
+        if (!few && W != fit32 && (W & 3u || W < 24)) continue;
+        const double t = rounds(W) * (W + fixed) * (W > 24 && K > (short_tables ? 64u : 32u) ? 1.05 : 1.0);
+        if (t < cost) {
+            cost = t;
+            best = ManyChains{32, W};
+        }
+    }
+    uint32_t G = 32, most = 32;  // fewer lanes: how many, and the most warps that pay
+    if (metropolis) {
+        if (npad <= (short_tables ? 512u : 256u)) G = 16;
+    } else if (K <= 32u) {
+        if (pm1 && npad <= 256u) G = 8, most = 16;
+    } else if (K <= 64u) {
+        if (npad <= (!pm1 ? 640u : short_tables ? 512u : 256u)) G = 16, most = pm1 ? 32 : 24;
+    } else if (K <= 128u) {
+        if (npad <= (pm1 && !short_tables ? 768u : 640u)) G = 16, most = 24;
+    }
+    if (G == 32) return best;
+    const uint32_t spw = 32 / G;
+    const uint32_t fit = std::min(most, fit_warps(per_chain, G));
+    for (uint32_t W = fit; W > (!few ? fit - 1u : G == 8 ? 15u : 16u); --W) {
+        const double t = rounds(spw * W) * (G == 8 ? 66.0 : 0.42 * spw * W + (most > 24 ? 35.0 : 22.0));
+        if (t < cost) {
+            cost = t;
+            best = ManyChains{G, W};
+        }
+    }
+    return best;
+}
+
 // Work items of the batch, grouped by launch class, each class with its own
 // lanes per chain and warps per CTA: the autotuned or forced values, else
 // the fewest lanes K allows (whole-warp chains for runs of few chains, where
@@ -1590,7 +1677,18 @@ sk_status plan_batch(sk_batch* b) {
         bool single = true;  // every run of the class has one chain: no overlap pairs
         for (uint32_t i : g.second) single = single && b->runs[i]->chains == 1;
         auto t = b->tuned.find(c.key);
-        if (t != b->tuned.end()) {
+        bool sum32 = false;
+        ManyChains many;
+        if (t == b->tuned.end() && !nw && !b->G_override && !b->S_override && !b->W_override && !b->C_override)
+            many = many_chains_layout(b, g.second, c.per_chain_direct, sms);
+        if (many.G) {
+            c.stage = 0;
+            c.G = many.G;
+            c.W = many.W;
+            c.per_chain = c.per_chain_direct;
+            // results of a Gaussian run do not depend on the default's lanes
+            sum32 = c.G == 16 && r0->inst->kind == SK_J_GAUSS;
+        } else if (t != b->tuned.end()) {
             c.stage = (t->second >> 16) & 0xFFu;
             c.G = (t->second >> 8) & 0xFFu;
             c.W = t->second & 0xFFu;
@@ -1627,7 +1725,8 @@ sk_status plan_batch(sk_batch* b) {
         }
         if (c.W < 1 || (c.G == 32 && c.W < 2 && !single))
             return fail(SK_ERR_INVALID_ARG, "N too large: %u bytes of shared memory per chain", c.per_chain);
-        c.cls = sk::step_class(r0->inst->kind, r0->p.rule, r0->p.K, c.G, nw ? 2u : c.stage, r0->inst->Npad);
+        c.cls = sk::step_class(r0->inst->kind, r0->p.rule, r0->p.K, c.G, nw ? 2u : sum32 ? 3u : c.stage,
+                               r0->inst->Npad);
         if (c.cls < 0) return fail(SK_ERR_INVALID_ARG, "no step kernel for K = %u with %u lanes per chain", r0->p.K, c.G);
         int occ = sk::step_kernel_occupancy(c.cls, c.W, c.per_chain);
         while (occ <= 0 && t == b->tuned.end() && c.W > (c.G == 32 ? 2u : 1u)) {  // default choice: step down
@@ -1641,7 +1740,7 @@ sk_status plan_batch(sk_batch* b) {
         for (uint32_t i : g.second) {
             const sk_run* r = b->runs[i];
             for (uint32_t ch = 0; ch < r->chains; ch += cpc)
-                items.push_back(WorkItem{i, ch, std::min(cpc, r->chains - ch), 0});
+                items.push_back(WorkItem{i, ch, std::min(cpc, r->chains - ch), sum32 ? sk::kItemSum32 : 0u});
         }
         c.n_items = static_cast<uint32_t>(items.size()) - c.first_item;
         c.grid = std::min<uint32_t>(c.n_items, static_cast<uint32_t>(occ * sms));

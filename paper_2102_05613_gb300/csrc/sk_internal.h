@@ -59,15 +59,21 @@ struct alignas(16) JobDev {
     // they write the spins back, so that the periodic recompute needs no
     // conversion; null when the run does not recompute periodically
     void* s_op;
-    uint64_t pad_;
+    // set by the step kernel in its copy, from the work item: 16-lane Gaussian
+    // chains add their weights and record energies as whole-warp chains do
+    uint32_t sum32;
+    uint32_t pad_;
 };
 static_assert(sizeof(JobDev) % 16 == 0, "JobDev is copied as 16-byte words");
 
 // A block of consecutive chains of one run, processed by one CTA (G lanes
 // per chain).  chain0 is even so that overlap pairs stay inside a CTA.
+// pad: the fused launch's variant and shared bytes; kItemSum32 for the step
+// kernel.
 struct WorkItem {
     uint32_t job, chain0, nchains, pad;
 };
+constexpr uint32_t kItemSum32 = 1;
 
 // Shared memory of the block-0 draws one chain keeps (16 bytes for each of
 // up to 32 steps).

@@ -44,6 +44,9 @@ int occupancy_pm1_metropolis_direct_nw(int, int, uint32_t, uint32_t);
 cudaError_t launch_step_gauss_mcmcmc_direct_nw(int, int, const JobDev*, const WorkItem*, uint32_t, uint32_t*,
                                       uint32_t, uint32_t, uint32_t, uint32_t, cudaStream_t);
 int occupancy_gauss_mcmcmc_direct_nw(int, int, uint32_t, uint32_t);
+cudaError_t launch_step_gauss_mcmcmc_direct_sum32(int, int, const JobDev*, const WorkItem*, uint32_t, uint32_t*,
+                                      uint32_t, uint32_t, uint32_t, uint32_t, cudaStream_t);
+int occupancy_gauss_mcmcmc_direct_sum32(int, int, uint32_t, uint32_t);
 cudaError_t launch_step_gauss_metropolis_direct_nw(int, int, const JobDev*, const WorkItem*, uint32_t, uint32_t*,
                                       uint32_t, uint32_t, uint32_t, uint32_t, cudaStream_t);
 int occupancy_gauss_metropolis_direct_nw(int, int, uint32_t, uint32_t);
@@ -500,7 +503,9 @@ int step_class(uint32_t kind, uint32_t rule, uint32_t K, uint32_t G, uint32_t st
     int lg = 0;
     while ((1u << lg) < G) ++lg;
     const int lnb = nb == 1 ? 0 : (nb == 2 ? 1 : 2);
-    return static_cast<int>(kind) * 256 + static_cast<int>(rule) * 128 + static_cast<int>(stage > 2 ? 0 : stage) * 32 +
+    // (3, the whole-warp order of sums: where the lanes' blocks make a difference)
+    if (stage > 2 && !(stage == 3 && kind == 1 && rule == 0 && nb == 2 && G == 16)) stage = 0;
+    return static_cast<int>(kind) * 256 + static_cast<int>(rule) * 128 + static_cast<int>(stage) * 32 +
            lnb * 8 + lg;
 }
 uint32_t class_lanes(int cls) { return 1u << (cls & 7); }
@@ -517,7 +522,8 @@ bool class_staged(int cls) { return ((cls >> 5) & 3) == 1; }
                  : stage_ == 2 ? F##_pm1_metropolis_direct_nw(__VA_ARGS__) : F##_pm1_metropolis_direct(__VA_ARGS__); \
         if (rule_ == 0)                                                              \
             return stage_ == 1 ? F##_gauss_mcmcmc_staged(__VA_ARGS__)                \
-                 : stage_ == 2 ? F##_gauss_mcmcmc_direct_nw(__VA_ARGS__) : F##_gauss_mcmcmc_direct(__VA_ARGS__); \
+                 : stage_ == 2 ? F##_gauss_mcmcmc_direct_nw(__VA_ARGS__)                                       \
+                 : stage_ == 3 ? F##_gauss_mcmcmc_direct_sum32(__VA_ARGS__) : F##_gauss_mcmcmc_direct(__VA_ARGS__); \
         return stage_ == 1 ? F##_gauss_metropolis_staged(__VA_ARGS__)                \
              : stage_ == 2 ? F##_gauss_metropolis_direct_nw(__VA_ARGS__) : F##_gauss_metropolis_direct(__VA_ARGS__); \
     } while (0)

@@ -392,10 +392,12 @@ __device__ __forceinline__ void update_fields(typename Types<JT>::H* hf, const J
     }
 }
 
-// E = -scale/2 sum_k s_k h_k of the group's chain.
+// E = -scale/2 sum_k s_k h_k of the group's chain.  sum32 (Gaussian, 16
+// lanes): bit for bit the whole-warp sum, lane l holding the partial sums of
+// that form's lanes l and l + 16.
 template <typename JT, int G>
 __device__ __forceinline__ double chain_energy(const int8_t* S, const void* h, uint32_t npad, double scale,
-                                               const Grp<G>& g) {
+                                               const Grp<G>& g, bool sum32 = false) {
     if constexpr (sizeof(JT) == 1) {
         const int* hf = static_cast<const int*>(h);
         int acc = 0;
@@ -411,16 +413,24 @@ __device__ __forceinline__ double chain_energy(const int8_t* S, const void* h, u
         // exact; relative rounding ~ (npad/G) 2^-24), the lanes' partial sums
         // are combined in double precision (FP64 is slow on this part)
         const float* hf = static_cast<const float*>(h);
-        float acc = 0.0f;
-        for (uint32_t k = 4u * g.gl; k < npad; k += 4u * G) {
-            const uint32_t sw = *reinterpret_cast<const uint32_t*>(S + k);
-            const float4 hv = *reinterpret_cast<const float4*>(hf + k);
-            acc = fmaf(static_cast<float>(sbyte(sw, 0)), hv.x, acc);
-            acc = fmaf(static_cast<float>(sbyte(sw, 1)), hv.y, acc);
-            acc = fmaf(static_cast<float>(sbyte(sw, 2)), hv.z, acc);
-            acc = fmaf(static_cast<float>(sbyte(sw, 3)), hv.w, acc);
-        }
-        return -0.5 * scale * gsum(g, static_cast<double>(acc));
+        auto partial = [&](uint32_t first, uint32_t stride) -> float {
+            float acc = 0.0f;
+            for (uint32_t k = first; k < npad; k += stride) {
+                const uint32_t sw = *reinterpret_cast<const uint32_t*>(S + k);
+                const float4 hv = *reinterpret_cast<const float4*>(hf + k);
+                acc = fmaf(static_cast<float>(sbyte(sw, 0)), hv.x, acc);
+                acc = fmaf(static_cast<float>(sbyte(sw, 1)), hv.y, acc);
+                acc = fmaf(static_cast<float>(sbyte(sw, 2)), hv.z, acc);
+                acc = fmaf(static_cast<float>(sbyte(sw, 3)), hv.w, acc);
+            }
+            return acc;
+        };
+        double mine;
+        if (G == 16 && sum32)
+            mine = static_cast<double>(partial(4u * g.gl, 128u)) + static_cast<double>(partial(4u * g.gl + 64u, 128u));
+        else
+            mine = static_cast<double>(partial(4u * g.gl, 4u * G));
+        return -0.5 * scale * gsum(g, mine);
     }
 }
 
@@ -542,7 +552,7 @@ __device__ __noinline__ void record(const JobDev& jb, bool write, uint32_t chain
     const Grp<G> g;
     const int8_t* partner_s = S + partner_off;
     const bool store = write && rec < jb.rec_capacity;
-    const double E = write ? chain_energy<JT, G>(S, h, jb.Npad, jb.scale, g) : 0.0;
+    const double E = write ? chain_energy<JT, G>(S, h, jb.Npad, jb.scale, g, jb.sum32 != 0u) : 0.0;
     // node-weighted energy of this state with the graph of the next step
     // (kernels built for runs that record it; groups without a chain skip it)
     double dm = 0.0;
@@ -586,6 +596,8 @@ __device__ __noinline__ void record(const JobDev& jb, bool write, uint32_t chain
 // rows through L1): the sites come in batches of G / SL steps (draw_site_batch; whole-warp
 // chains hold one slot per lane), and for +-J the slot-weight scan covers
 // only the lanes that hold slots (the integer total is the same in any order).
+// STAGE 3 (Gaussian, 16 lanes with two blocks each): the weights are added in
+// the whole-warp form's order, so that the two layouts choose alike.
 template <typename JT, int RULE, int NB, int G, int STAGE, int UNROLL, bool RCH, bool FAST = false, int SL = 0>
 __device__ __forceinline__ void chain_loop(const JobDev& jb, bool write, uint32_t chain, const ChainMem& cm,
                                            int partner_off, uint32_t t0, uint32_t t1, uint32_t& acc,
@@ -594,6 +606,7 @@ __device__ __forceinline__ void chain_loop(const JobDev& jb, bool write, uint32_
     using W = typename Types<JT>::W;
     constexpr bool STAGED = STAGE == 1;  // 0: rows through L1, 2: the same with node-weighted records
     constexpr bool NWR = STAGE == 2;
+    constexpr bool SUM32 = STAGE == 3;
     // the 128-register variant (few warps per SM, where one chain's step is a
     // chain of latencies) keeps the slot weights in registers for the node
     // search and draws the next step's sites during the current step
@@ -894,8 +907,29 @@ __device__ __forceinline__ void chain_loop(const JobDev& jb, bool write, uint32_
                 }
                 W incl[NB], tot[NB];
                 W total = w0;
+                if constexpr (SUM32) {
+                    // block q of lane l is lane l + 16 q of the whole-warp
+                    // scan: its levels 1 to 8 rotate within the 16 lanes
+                    // (block 1 takes from block 0 across the wrap), level 16
+                    // adds block 0 to block 1: 9 shuffles for the two chains of
+                    // a warp, where two whole-warp chains take 12.
+                    static_assert(sizeof(JT) == 4 && NB == 2 && G == 16, "Gaussian, two blocks on 16 lanes");
+                    W v0 = gsum_[0], v1 = gsum_[1];
 #pragma unroll
-                for (int q = 0; q < NB; ++q) {
+                    for (int o = 1; o < G; o <<= 1) {
+                        const W y0 = gshfl(g, v0, (g.gl - o) & (G - 1));
+                        const W y1 = gshfl(g, v1, (g.gl - o) & (G - 1));
+                        v1 += g.gl >= o ? y1 : y0;
+                        if (g.gl >= o) v0 += y0;
+                    }
+                    incl[0] = v0;
+                    incl[1] = v1 + v0;
+                    tot[0] = 0;  // block 1's prefixes hold block 0
+                    tot[1] = gshfl(g, incl[1], G - 1);
+                    total += tot[1];
+                }
+#pragma unroll
+                for (int q = 0; q < (SUM32 ? 0 : NB); ++q) {
                     if constexpr (PAIRS) {  // over the 16 odd lanes (the even ones' values are not used)
                         W v = gsum_[0];
 #pragma unroll
@@ -1280,7 +1314,9 @@ __device__ __forceinline__ void run_item(const WorkItem& wi, const JobDev& jb, u
 // (65536 / MAXT): 1024 -> 64, 768 -> 80, 640 -> 96, 512 -> 128 registers.
 // STAGE: 1 stages row a by TMA (two row buffers per chain in shared memory),
 // 0 reads it through L1 (no buffers: more chains fit in shared memory), 2 is
-// 0 with node-weighted energy records (for runs that ask for them).
+// 0 with node-weighted energy records (for runs that ask for them), 3 is 0 with
+// the weights added in the whole-warp order (16 lanes; a kernel of its own, as
+// a second loop in kernel 0 cost that one 2 %).
 template <typename JT, int RULE, int NB, int G, int STAGE, int MAXT, bool RCH = false>
 __global__ void __launch_bounds__(MAXT, 1)
     step_kernel(const JobDev* __restrict__ jobs, const WorkItem* __restrict__ items, uint32_t n_items,
@@ -1312,6 +1348,10 @@ __global__ void __launch_bounds__(MAXT, 1)
             reinterpret_cast<uint4*>(&s_job)[threadIdx.x] = reinterpret_cast<const uint4*>(&jobs[wi.job])[threadIdx.x];
         __syncthreads();
         const JobDev& jb = s_job;
+        if constexpr (sizeof(JT) == 4 && G == 16) {
+            if (threadIdx.x == 0) s_job.sum32 = wi.pad & kItemSum32;
+            __syncthreads();
+        }
         if constexpr (sizeof(JT) == 1) {  // the start of the +-J weight table (0 past its end)
             for (uint32_t i = threadIdx.x; i < kWCache; i += blockDim.x)
                 s_wt[i] = i < jb.wlen ? reinterpret_cast<const unsigned long long*>(jb.W)[i] : 0ull;

@@ -269,3 +269,27 @@ def test_recompute_on_256_row_tiles(N, chains):
     h2 = state()[1]
     assert torch.equal(h1, h2) and st["max_field_drift"] == 0.0 and (h2.double() - exact).abs().max().item() <= tol
     run.close(); inst.close()
+
+
+@pytest.mark.parametrize("rule,K,N", [(0, 33, 77), (0, 64, 640), (0, 65, 33), (0, 100, 512), (0, 128, 130), (1, 1, 250)])
+def test_default_layout_of_many_chains(rule, K, N):
+    # Gaussian chains beyond 32 per SM default to 16 lanes with the whole-warp
+    # form's sums: every result (trace, records with their energies, state)
+    # bit for bit that of forced whole warps; ragged N, K and last item
+    torch = need_gpu()
+    chains = 33 * torch.cuda.get_device_properties(0).multi_processor_count + 1
+    J = inputs.couplings(N, sk.SK_J_GAUSS, 71)
+    init = inputs.initial_spins(chains, N, 72)
+    outs = []
+    for lanes in (0, 32):
+        inst = sk.Instance(J)
+        run = sk.Run(inst, chains=chains, K=K, rule=rule, beta=1.2, seed=73, record_every=16, max_records=3, init=init,
+                     trace_chains=chains, trace_steps=48, p_center=0.2 if K == 100 else 0.0)
+        b = sk.Batch([run])
+        b.set_layout(lanes=lanes)
+        assert b.classes()[0][1] == (lanes or 16)
+        for n in (1, 16, 31):
+            b.advance(n)
+        outs.append((run.trace(),) + run.observables() + run.state(fields=True) + run.counters())
+        b.close(); run.close(); inst.close()
+    assert all(np.array_equal(x, y) for x, y in zip(*outs))
