@@ -31,6 +31,7 @@
 #include <stdint.h>
 
 #include <algorithm>
+#include <numeric>
 #include <cstring>
 #include <mutex>
 #include <set>
@@ -846,7 +847,12 @@ cudaError_t launch_set_fields_batch(uint32_t kind, const RecomputeSet* sets, uin
         kb += b.args.terms * b.args.kblocks;
     }
     const bool tall = bf && tall_tiles(nt1, nt2, static_cast<uint32_t>(kb / n), false);
-    for (uint32_t i = 0; i < n; ++i)
+    // longest tiles first: CTA c takes tasks c, c + grid, ..., and the sets may
+    // differ in N (mixed order would leave the last round to the long ones)
+    std::vector<uint32_t> order(n);
+    std::iota(order.begin(), order.end(), 0u);
+    std::stable_sort(order.begin(), order.end(), [&](uint32_t x, uint32_t y) { return sets[x].npad > sets[y].npad; });
+    for (uint32_t i : order)
         for (uint32_t m0 = 0; m0 < sets[i].chains; m0 += tall ? 2 * BM : BM)
             for (uint32_t n0 = 0; n0 < sets[i].npad; n0 += BN) tasks.push_back(BatchTask{i, m0, n0, 0});
     SegSpins* dseg = nullptr;

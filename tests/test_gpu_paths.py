@@ -293,3 +293,28 @@ def test_default_layout_of_many_chains(rule, K, N):
         outs.append((run.trace(),) + run.observables() + run.state(fields=True) + run.counters())
         b.close(); run.close(); inst.close()
     assert all(np.array_equal(x, y) for x, y in zip(*outs))
+
+
+def test_reset_many_by_stream_and_kind():
+    # runs of both coupling kinds, uneven sizes and two streams restarted in one
+    # call (grouped by stream and kind, one run alone) against single restarts
+    torch = need_gpu()
+    sts = [torch.cuda.Stream(), torch.cuda.Stream()]
+    specs = [(33, 0, 6, 0), (700, 1, 300, 0), (200, 0, 258, 0), (64, 1, 1, 0), (1024, 1, 130, 0), (96, 0, 10, 1)]
+    insts = [sk.Instance(inputs.couplings(N, k, 600 + i), stream=sts[s]) for i, (N, k, _, s) in enumerate(specs)]
+    inits = [inputs.initial_spins(c, N, 700 + i) for i, (N, _, c, _) in enumerate(specs)]
+    inits[2] = None
+    runs = [sk.Run(x, chains=c, K=8, seed=2, stream_id=i, record_every=10, max_records=2)
+            for i, (x, (_, _, c, _)) in enumerate(zip(insts, specs))]
+    for r in runs:
+        r.advance(20)
+    sk.reset_many(runs, inits)
+    got = [r.state(fields=True) + r.observables() + r.counters() for r in runs]
+    for i, r in enumerate(runs):
+        r.advance(10)
+        r.reset(inits[i])
+        one = r.state(fields=True) + r.observables() + r.counters()
+        assert one[2] == 0 and all(np.array_equal(x, y) for x, y in zip(got[i], one)), i
+        r.close()
+    for x in insts:
+        x.close()
