@@ -418,8 +418,10 @@ sk_status mcmcmc_batch_autotune(sk_batch* b, uint32_t trial_steps, uint32_t* war
  *            0 = default: whole-warp chains (32 lanes), or for star classes
  *            the team layout of 2 or 4 warps per chain (64 / 128 lanes below)
  *            where the batch's chains are few enough to run in one round of
- *            its CTAs, and for graph classes the warps per chain that finish
- *            the class's chains first; a value that
+ *            its CTAs, 16 or 8 lanes where they exceed 32 per SM and N and K
+ *            make those faster (Gaussian chains there repeat the whole-warp
+ *            results bit for bit), and for graph classes the warps per chain
+ *            that finish the class's chains first; a value that
  *            leaves no room for one warp's chains in a CTA's shared memory
  *            is raised until they fit.  Kernels exist
  *            for 1 block per lane at every width, 2 blocks at 8, 16 and 32
