@@ -1204,9 +1204,9 @@ sk_status mcmcmc_recompute(sk_run* r, uint32_t mode, uint32_t terms, sk_recomput
     float* dout = nullptr;
     if (mode == 2 && (s = dalloc(&dout, static_cast<size_t>(r->chains) * in->Npad * 4)) != SK_OK) return s;
     SK_CU(cudaMemsetAsync(r->dstats + 3, 0, 3 * sizeof(unsigned long long), st));
-    // a resynchronisation of Gaussian fields whose figures nobody gets only
-    // sets the fields: it need not read the old ones and the spins
-    const uint32_t kmode = mode == 1 && !stats && in->kind == SK_J_GAUSS ? 3u : mode;
+    // a resynchronisation whose figures nobody gets only sets the fields: it
+    // need not read the old ones and the spins
+    const uint32_t kmode = mode == 1 && !stats ? 3u : mode;
     cudaError_t e = sk::launch_recompute(in->kind, r->ds, r->dh, dout, r->dSop, in->dJop, r->ddE, r->dstats + 3,
                                          r->derr, r->chains, in->Npad, terms ? terms : 3u, kmode, in->scale, st,
                                          r->job.fault & sk::kFaultWithholdTile, r->sop_valid, r->dCnt);

@@ -208,6 +208,17 @@ __device__ __forceinline__ void load_row_block(RowBlock& rb, const Args& args, u
         rb.s[1] = __ldg(sp + 1);
     }
 }
+// Four accumulator values as maintained fields: int32 for +-J, float32 else.
+__device__ __forceinline__ uint4 field_words(const uint32_t (&v)[32], int q, uint32_t pm1) {
+    uint4 w = make_uint4(v[4 * q], v[4 * q + 1], v[4 * q + 2], v[4 * q + 3]);
+    if (pm1) {
+        w.x = static_cast<uint32_t>(__float2int_rn(__uint_as_float(w.x)));
+        w.y = static_cast<uint32_t>(__float2int_rn(__uint_as_float(w.y)));
+        w.z = static_cast<uint32_t>(__float2int_rn(__uint_as_float(w.z)));
+        w.w = static_cast<uint32_t>(__float2int_rn(__uint_as_float(w.w)));
+    }
+    return w;
+}
 // first: the first column block, loaded by the caller (before it waited for
 // the accumulator) with load_row_block(first, args, row0 + lane, n0 + c0, ..).
 __device__ __forceinline__ void epilogue_rows(uint32_t taddr, const Args& args, uint32_t row0, uint32_t n0,
@@ -233,16 +244,9 @@ __device__ __forceinline__ void epilogue_rows(uint32_t taddr, const Args& args, 
             uint4* dst = args.mode == 2 ? reinterpret_cast<uint4*>(args.out + idx)
                                         : reinterpret_cast<uint4*>(static_cast<unsigned int*>(args.h) + idx);
 #pragma unroll
-            for (int q = 0; q < 8; ++q) {
-                uint4 w = make_uint4(v[4 * q], v[4 * q + 1], v[4 * q + 2], v[4 * q + 3]);
-                if (args.mode == 3 && args.pm1) {
-                    w.x = static_cast<uint32_t>(__float2int_rn(__uint_as_float(w.x)));
-                    w.y = static_cast<uint32_t>(__float2int_rn(__uint_as_float(w.y)));
-                    w.z = static_cast<uint32_t>(__float2int_rn(__uint_as_float(w.z)));
-                    w.w = static_cast<uint32_t>(__float2int_rn(__uint_as_float(w.w)));
-                }
-                dst[q] = w;
-            }
+            for (int q = 0; q < 8; ++q)
+                dst[q] = args.mode == 3 ? field_words(v, q, args.pm1)
+                                        : make_uint4(v[4 * q], v[4 * q + 1], v[4 * q + 2], v[4 * q + 3]);
             continue;
         }
 #pragma unroll
@@ -264,7 +268,7 @@ __device__ __forceinline__ void epilogue_rows(uint32_t taddr, const Args& args, 
         if (args.mode == 1) {  // resync: the maintained fields become H
             uint4* dst = reinterpret_cast<uint4*>(static_cast<unsigned int*>(args.h) + idx);
 #pragma unroll
-            for (int q = 0; q < 8; ++q) dst[q] = make_uint4(v[4 * q], v[4 * q + 1], v[4 * q + 2], v[4 * q + 3]);
+            for (int q = 0; q < 8; ++q) dst[q] = field_words(v, q, args.pm1);
         }
     }
     if (tile_ok && reads) {
