@@ -470,7 +470,7 @@ __device__ __forceinline__ void chain_steps(const JobDev& jb, bool write, uint32
             for (int q = 0; q < NB; ++q) {
                 const unsigned ball = __ballot_sync(kFull, !found && base + incl[q] > u);
                 if (!found && ball) {
-                    const int L = __ffs(ball) - 1;
+                    int L = __ffs(ball) - 1;
                     W mine = 0;
 #pragma unroll
                     for (int e = 0; e < 4; ++e) mine += xs[4 * q + e];
@@ -487,16 +487,16 @@ __device__ __forceinline__ void chain_steps(const JobDev& jb, bool write, uint32
                         }
                     }
                     if (my_e < 0) my_e = last_pos;
-                    uint32_t my = 0;
+                    uint32_t my = step::kNoSlot;
 #pragma unroll
                     for (int e = 0; e < 4; ++e)
                         if (e == my_e)
                             my = (step::site_of<NB>(site, 4 * q + e) << 3) | (((sneg >> (4 * q + e)) & 1u) << 2) |
                                  static_cast<uint32_t>(e);
-                    const uint32_t packed = __shfl_sync(kFull, my, L);
+                    const uint32_t packed = step::owner_word(g, my, L, q);
+                    sel_d = 128 * q + 4 * L + static_cast<int>(packed & 3u) + 1;
                     sel_site = packed >> 3;
                     sel_neg = (packed >> 2) & 1u;
-                    sel_d = 128 * q + 4 * L + static_cast<int>(packed & 3u) + 1;
                     found = true;
                 }
                 base += tot[q];

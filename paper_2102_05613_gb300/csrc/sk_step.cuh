@@ -242,6 +242,30 @@ __device__ __forceinline__ uint32_t site_of(const uint32_t (&sp)[2 * NB], int k)
 __device__ __forceinline__ uint32_t site_pick(uint32_t w0, uint32_t w1, int e) {
     return (((e & 2) ? w1 : w0) >> (16 * (e & 1))) & 0xFFFFu;
 }
+// A lane's answer to the search of its weights: site << 2 | entry, all ones
+// where it has no positive weight.  The first lane L whose prefix exceeds u is
+// normally the owner; but sums are rounded, and the tree of the scan can give
+// a lane without a positive weight a prefix one rounding above that of the
+// last positive lane before it (Gaussian: ~2e-8 of the steps where K does not
+// fill the lanes).  The owner is then that last positive lane, and L becomes
+// it.  There is one where the scan starts in this block, as its prefixes are 0
+// up to the first; with none, L becomes -1 - G q, so that the slot of an
+// all-ones word, 4 G q + 4 L + 4, is 0, the root.  (One word of each lane kept
+// past the shuffle and one comparison: 0 to 1 % of a step, a lone chain's 1 to
+// 3 %; 8 x 8192 chains, N = 512, K = 128, 100 steps 4258 -> 4277 us.  With the
+// weights and sites kept for a second search the throughput variants lost 2 to 13 %.)
+constexpr uint32_t kNoSite = 0x3FFFFFFFu, kNoSlot = 0xFFFFFFFFu;
+template <int G>
+__device__ __forceinline__ uint32_t owner_word(const Grp<G>& g, uint32_t mine, int& L, int q) {
+    uint32_t word = gshfl(g, mine, L);
+    if (word == kNoSlot) {
+        const unsigned pos = gballot(g, mine != kNoSlot) & ((2u << L) - 1u);
+        L = pos ? 31 - __clz(pos) : -1 - G * q;
+        word = gshfl(g, mine, pos ? L : 0);
+        if (!pos) word = kNoSlot;
+    }
+    return word;
+}
 // The first of a lane's four weights whose prefix run + x[0] + .. exceeds u;
 // failing that (a rounding guard) its last positive one, -1 if there is none.  The prefixes are
 // taken one after the other, the comparisons side by side: a weight of 0 adds
@@ -982,11 +1006,11 @@ __device__ __forceinline__ void chain_loop(const JobDev& jb, bool write, uint32_
                 if constexpr (PAIRS) {
                     const unsigned over = gballot(g, !found && (g.gl & 1) && base + incl[0] > u);
                     if (over) {
-                        const int L = __ffs(over) - 1;
-                        const int my_e = first_past(x4, base + (incl[0] - gsum_[0]), u);
+                        int L = __ffs(over) - 1;
+                        const int my_e = (g.gl & 1) ? first_past(x4, base + (incl[0] - gsum_[0]), u) : -1;
                         const uint32_t my_site =
-                            my_e < 0 ? 0u : (((my_e & 2) ? site[0] : site_even) >> (16 * (my_e & 1))) & 0xFFFFu;
-                        const uint32_t packed = gshfl(g, (my_site << 2) | static_cast<uint32_t>(my_e & 3), L);
+                            my_e < 0 ? kNoSite : (((my_e & 2) ? site[0] : site_even) >> (16 * (my_e & 1))) & 0xFFFFu;
+                        const uint32_t packed = owner_word(g, (my_site << 2) | static_cast<uint32_t>(my_e & 3), L, 0);
                         sel_site = packed >> 2;
                         sel_d = 4 * (L >> 1) + static_cast<int>(packed & 3u) + 1;
                         found = true;
@@ -1040,11 +1064,11 @@ __device__ __forceinline__ void chain_loop(const JobDev& jb, bool write, uint32_
                             for (int q = 1; q < NB; ++q)
                                 if (q == qf) x[e] = xs[4 * q + e];
                         }
-                        const int L = __ffs(ball) - 1;
+                        int L = __ffs(ball) - 1;
                         W mine = 0;
 #pragma unroll
                         for (int e = 0; e < 4; ++e) mine += x[e];
-                        uint32_t my_site = 0;
+                        uint32_t my_site = kNoSite;
                         int my_e = -1;
                         if constexpr (LEAN) {
                             my_e = first_past(x, bse + (inc - mine), u);
@@ -1076,7 +1100,21 @@ __device__ __forceinline__ void chain_loop(const JobDev& jb, bool write, uint32_
                                 for (int e = 0; e < 4; ++e)
                                     if (q == qf && e == my_e) my_site = site_of<NB>(site, 4 * q + e);
                         }
-                        const uint32_t packed = gshfl(g, (my_site << 2) | static_cast<uint32_t>(my_e & 3), L);
+                        uint32_t packed = owner_word(g, (my_site << 2) | static_cast<uint32_t>(my_e & 3), L, qf);
+                        if constexpr (SUM32) {
+                            // (block 1's prefixes hold block 0's: the last
+                            // positive lane may be one of that block)
+                            if (L < 0) {
+                                qf = 0;
+                                L = G - 1;
+                                W x0[4], sum = 0;
+#pragma unroll
+                                for (int e = 0; e < 4; ++e) sum += x0[e] = xs[e];
+                                const int e0 = first_past(x0, w0 + (incl[0] - sum), u);
+                                packed = owner_word(
+                                    g, e0 < 0 ? kNoSlot : (site_pick(site[0], site[1], e0) << 2) | static_cast<uint32_t>(e0), L, 0);
+                            }
+                        }
                         sel_site = packed >> 2;
                         sel_d = 4 * G * qf + 4 * L + static_cast<int>(packed & 3u) + 1;
                         found = true;
@@ -1087,7 +1125,7 @@ __device__ __forceinline__ void chain_loop(const JobDev& jb, bool write, uint32_
                     const unsigned ball =
                         gballot(g, !found && base + incl[q] > u && (!SCANSL || g.gl < SCANL));
                     if (!found && ball) {
-                        const int L = __ffs(ball) - 1;
+                        int L = __ffs(ball) - 1;
                         // this lane's 4 weights (kept, or recomputed bit-identically),
                         // their sum in the order of the first pass
                         W x[4];
@@ -1100,7 +1138,7 @@ __device__ __forceinline__ void chain_loop(const JobDev& jb, bool write, uint32_
                                 x[e] = slot_w(4 * q + e);
                             mine += x[e];
                         }
-                        uint32_t my_site = 0;
+                        uint32_t my_site = kNoSite;
                         int my_e = -1;
                         if constexpr (LEAN) {
                             my_e = first_past(x, base + (incl[q] - mine), u);
@@ -1123,7 +1161,9 @@ __device__ __forceinline__ void chain_loop(const JobDev& jb, bool write, uint32_
                             for (int e = 0; e < 4; ++e)
                                 if (e == my_e) my_site = site_of<NB>(site, 4 * q + e);
                         }
-                        const uint32_t packed = gshfl(g, (my_site << 2) | static_cast<uint32_t>(my_e & 3), L);
+                        const uint32_t word = (my_site << 2) | static_cast<uint32_t>(my_e & 3);
+                        // (+-J sums are exact)
+                        const uint32_t packed = sizeof(JT) == 4 ? owner_word(g, word, L, q) : gshfl(g, word, L);
                         sel_site = packed >> 2;
                         sel_d = 4 * G * q + 4 * L + static_cast<int>(packed & 3u) + 1;
                         found = true;

@@ -330,7 +330,6 @@ __device__ __forceinline__ void team_loop(const JobDev& jb, bool write, uint32_t
             // every thread's weight, its slot's spin in the sign bit (a warp ahead
             // may flip spins before another gets to the choice)
             put_weight(&wx[tid], x, si);
-            if (tid == 0) put_weight(&wx[NT], W(0), S[0]);
             team_sync(bar, NT);  // 2: the weights
             // Every warp takes the same scan of all the slots' weights, in the
             // order of the one-warp layout: K <= 32 one slot per lane, else
@@ -359,8 +358,8 @@ __device__ __forceinline__ void team_loop(const JobDev& jb, bool write, uint32_t
             }
             if (!(u < w0)) {  // a slot d >= 1 (the same decision in every thread)
                 // the first lane whose prefix exceeds u; a rounding guard takes
-                // the last lane up to it with a positive weight (K <= 32), or
-                // the owning lane's last positive weight
+                // the last lane up to it with a positive weight, and there (K >
+                // 32) the owning lane's last positive weight
                 const unsigned over = __ballot_sync(kFull, w0 + incl > u);
                 int L = over ? __ffs(over) - 1 : 31;
                 uint32_t pick = 0;  // slot; bit 16: its spin is -1
@@ -370,22 +369,17 @@ __device__ __forceinline__ void team_loop(const JobDev& jb, bool write, uint32_t
                     pick = pos ? static_cast<uint32_t>(L) + 1u : 0u;
                     pick |= __shfl_sync(kFull, neg, L) << 16;
                 } else if (over) {
-                    const int my_e = step::first_past(wl, w0 + (incl - mine), u);
-                    const uint32_t q = static_cast<uint32_t>(my_e & 3);
-                    // bit 17: no positive weight there, the one-warp layout's site 0
-                    pick = __shfl_sync(kFull, (4u * lane + q + 1u) | (((neg >> q) & 1u) << 16) | (my_e < 0 ? 1u << 17 : 0u), L);
+                    const int e = step::first_past(wl, w0 + (incl - mine), u);
+                    pick = step::owner_word(
+                        g, e < 0 ? step::kNoSlot : (4u * lane + e + 1u) | (((neg >> e) & 1u) << 16), L, 0);
+                    if (pick == step::kNoSlot) pick = 0u;
                 }
                 sel = static_cast<int>(pick & 0xFFFFu);
                 if (sel != 0) {
                     const uint32_t q = static_cast<uint32_t>(sel) - 1u;
                     const uint2 es = rb[(q >> 2) & (SL - 1u)];
-                    uint32_t sel_site = step::site_pick(es.x, es.y, static_cast<int>(q & 3u));
-                    int s_b = (pick & 0x10000u) ? -1 : 1;
-                    if (pick >> 17) {
-                        W zero;
-                        sel_site = 0u;
-                        s_b = get_weight(&wx[NT], zero) ? -1 : 1;
-                    }
+                    const uint32_t sel_site = step::site_pick(es.x, es.y, static_cast<int>(q & 3u));
+                    const int s_b = (pick & 0x10000u) ? -1 : 1;
                     if (!leaf) {
                         nflip = 1;
                         x1 = sel_site;

@@ -38,3 +38,56 @@ def test_pm1_resync_sets_integer_fields(N, chains, figures):
     o = oracle.run(J, K=24, beta=0.7, seed=93, chains=chains, init=init, steps=40, record_every=20)
     assert np.array_equal(E, o["E"]) and np.array_equal(acc, o["acc"]) and np.array_equal(run.state()[0], o["spins"])
     run.close(); inst.close()
+
+
+# Gaussian, N = 64, couplings seed 81, starts seed 82, beta = 1: (K, run seed, chain, step) where the
+# draw lies between the last slot's prefix and the rounded total.
+GAPS = [(40, 144, 300, 859), (40, 24, 1746, 72), (100, 119, 919, 917), (100, 98, 1729, 448), (200, 58, 902, 838),
+        (200, 64, 2170, 398)]
+
+
+@pytest.mark.parametrize("K,seed,chain,step", GAPS)
+def test_search_never_leaves_the_slots(K, seed, chain, step):
+    # the search took slot 4 L + 4 (past K) with site 0 there, unproposed; now
+    # the last slot with a positive weight, alike in every layout
+    need_gpu()
+    N, steps = 64, step + 20
+    J = inputs.couplings(N, sk.SK_J_GAUSS, 81)
+    init = inputs.initial_spins(4900, N, 82)
+
+    def go(chains, warps=0, lanes=0, staging=0, cluster=0, fused=0):
+        inst = sk.Instance(J)
+        run = sk.Run(inst, chains=chains, K=K, beta=1.0, seed=seed, init=init[:chains], trace_chains=chains,
+                     trace_steps=steps)
+        b = sk.Batch([run], warps_per_cta=warps)
+        if lanes or staging:
+            b.set_layout(lanes=lanes, staging=staging)
+        if cluster:
+            b.set_cluster(cluster)
+        if fused:
+            b.set_fused(fused)
+        b.advance(steps)
+        out = run.trace(), run.state(fields=True)
+        b.close(); run.close(); inst.close()
+        return out
+
+    few = chain + 1
+    forms = [dict(chains=4900), dict(chains=few), dict(chains=few, warps=4, lanes=32, staging=2),
+             dict(chains=few, warps=24, lanes=32, staging=2), dict(chains=few, warps=4, lanes=32, staging=1),
+             dict(chains=few, cluster=1), dict(chains=few, cluster=2), dict(chains=few, fused=8)]
+    if K <= 128:
+        forms.append(dict(chains=few, lanes=128))
+    if K <= 64:
+        forms += [dict(chains=few, lanes=64), dict(chains=few, lanes=16, staging=2)]
+    tr0, (s0, h0, _) = go(**forms[0])
+    assert tr0.max() <= K and tr0[chain, step] == K
+    r = oracle.replay(J, tr0[chain], K=K, beta=1.0, seed=seed, chain=chain, init=init[chain], tol=1e-4)
+    assert r["bad"] == 0 and np.array_equal(r["spins"], s0[chain])
+    for f in forms[1:]:
+        tr, (s, h, _) = go(**f)
+        n = f["chains"]
+        assert np.array_equal(tr, tr0[:n]) and np.array_equal(s, s0[:n]) and np.array_equal(h, h0[:n]), f
+    # layouts with sums of their own
+    for lanes in (8, 16):
+        if K <= 16 * lanes:
+            assert go(few, lanes=lanes, staging=2)[0].max() <= K
