@@ -12,7 +12,9 @@
 #include <cstdio>
 #include <cstring>
 #include <map>
+#include <memory>
 #include <mutex>
+#include <new>
 #include <string>
 #include <thread>
 #include <vector>
@@ -744,6 +746,9 @@ sk_status sk_energy(const sk_instance* in, const int8_t* spins, uint32_t count, 
     const bool check_here = host && n <= 16384;
     for (size_t i = 0; check_here && i < n; ++i)
         if (spins[i] != 1 && spins[i] != -1) return fail(SK_ERR_INVALID_ARG, "spin %zu is not +-1", i);
+    // the energies on the host until nothing can fail any more
+    std::unique_ptr<double[]> hE(new (std::nothrow) double[count]);
+    if (!hE) return fail(SK_ERR_OOM, "no host memory for %u energies", count);
     auto up = [](size_t b) { return (b + 1023u) & ~static_cast<size_t>(1023u); };
     // workspace: the result of the spins' check, the energies, the column
     // parts of the direct sum, host spins, the tensor path's operands
@@ -763,7 +768,6 @@ sk_status sk_energy(const sk_instance* in, const int8_t* spins, uint32_t count, 
     unsigned long long* dflag = reinterpret_cast<unsigned long long*>(base);
     double* dE = reinterpret_cast<double*>(base + o_E);
     const int8_t* dsp = spins;
-    std::vector<double> hE(count);
     unsigned long long hflag = ~0ull;
     int herr = 0;
     cudaError_t e = cudaSuccess;
@@ -783,7 +787,7 @@ sk_status sk_energy(const sk_instance* in, const int8_t* spins, uint32_t count, 
     if (e == cudaSuccess && !(tc && in->kind == SK_J_PM1))  // (Gaussian: writes only if the launch above did not)
         e = sk::launch_energy(in->dJ, in->kind, in->N, in->Npad, in->scale, dsp, count, dE, in->st,
                               tiles > 1 ? reinterpret_cast<double*>(base + o_part) : nullptr, slices);
-    if (e == cudaSuccess) e = cudaMemcpyAsync(hE.data(), dE, count * sizeof(double), cudaMemcpyDeviceToHost, in->st);
+    if (e == cudaSuccess) e = cudaMemcpyAsync(hE.get(), dE, count * sizeof(double), cudaMemcpyDeviceToHost, in->st);
     if (e == cudaSuccess && err) e = cudaMemcpyAsync(&herr, err, sizeof herr, cudaMemcpyDeviceToHost, in->st);
     cudaFreeAsync(ws, in->st);
     const cudaError_t e2 = cudaStreamSynchronize(in->st);
@@ -791,7 +795,7 @@ sk_status sk_energy(const sk_instance* in, const int8_t* spins, uint32_t count, 
     if (e != cudaSuccess) return fail(SK_ERR_CUDA, "sk_energy: %s", cudaGetErrorString(e));
     if (hflag != ~0ull) return fail(SK_ERR_INVALID_ARG, "spin %llu is not +-1", hflag >> 2);
     if (herr) return fail(SK_ERR_TIMEOUT, "sk_energy: a bounded device wait expired");
-    std::memcpy(out_E, hE.data(), count * sizeof(double));
+    std::memcpy(out_E, hE.get(), count * sizeof(double));
     return SK_OK;
 }
 

@@ -1,4 +1,8 @@
 """Results that single paths once got wrong: each test fails on the form it names."""
+import os
+import subprocess
+import sys
+
 import numpy as np
 import pytest
 
@@ -8,6 +12,7 @@ from paper_2102_05613_gb300 import inputs, sk
 from gpu_util import need_gpu
 
 pytestmark = pytest.mark.gpu
+ROOT = os.path.dirname(os.path.dirname(os.path.abspath(__file__)))
 
 
 @pytest.mark.parametrize("figures", [True, False])
@@ -91,3 +96,32 @@ def test_search_never_leaves_the_slots(K, seed, chain, step):
     for lanes in (8, 16):
         if K <= 16 * lanes:
             assert go(few, lanes=lanes, staging=2)[0].max() <= K
+
+
+def test_energy_without_host_memory_is_an_error():
+    # the host copy of the energies threw through the C entry and ended the
+    # process; in a process of its own whose data size is limited meanwhile
+    need_gpu()
+    code = """
+import ctypes as C, resource, sys
+import numpy as np, torch
+from paper_2102_05613_gb300 import inputs, sk
+count = 1 << 25
+s = torch.ones((count, 2), dtype=torch.int8, device="cuda")
+out = np.zeros(count)
+inst = sk.Instance(inputs.couplings_pm1(2, 1))
+def call(n):
+    return sk.lib().sk_energy(inst.handle, C.c_void_p(s.data_ptr()), n, sk.SK_MEM_DEVICE,
+                              out.ctypes.data_as(C.c_void_p))
+assert call(1000) == sk.SK_OK
+data = [int(x.split()[1]) for x in open("/proc/self/status") if x.startswith("VmData")][0] << 10
+soft, hard = resource.getrlimit(resource.RLIMIT_DATA)
+resource.setrlimit(resource.RLIMIT_DATA, (data + (100 << 20), hard))
+st = call(count)
+resource.setrlimit(resource.RLIMIT_DATA, (soft, hard))
+assert st == sk.SK_ERR_OOM and not out[1000:].any(), st
+assert call(count) == sk.SK_OK and np.all(out == out[0]) and abs(out[0]) == 1.0
+inst.close()
+"""
+    r = subprocess.run([sys.executable, "-c", code], cwd=ROOT, capture_output=True, text=True, timeout=300)
+    assert r.returncode == 0, r.stderr[-2000:]
