@@ -66,14 +66,25 @@ sk_status check_device() {
     return SK_OK;
 }
 
+template <typename T>
+sk_status dalloc(T** p, size_t bytes) {
+    *p = nullptr;
+    if (bytes == 0) return SK_OK;
+    cudaError_t e = cudaMalloc(reinterpret_cast<void**>(p), bytes);
+    if (e != cudaSuccess) {
+        cudaGetLastError();
+        return fail(SK_ERR_OOM, "cudaMalloc(%zu) failed: %s", bytes, cudaGetErrorString(e));
+    }
+    return SK_OK;
+}
+
 // Stream-ordered workspace of calls that need some only while they run, from
 // one memory pool per device: up to kWorkspaceKept bytes stay with the pool
 // between calls (a cudaMalloc / cudaFree pair of the 80 MB an energy call at
 // N = 2048 takes costs more than its kernels), more goes back at the next
 // synchronisation, and all of it when the process's last instance is
-// destroyed (set generation, which needs no instance, takes less than 1 MB) or
-// a device allocation of the library finds no room.  The runtime's pools are
-// safe for concurrent threads and order reuse between streams.
+// destroyed.  The runtime's pools are safe for concurrent threads and order
+// reuse between streams.
 constexpr uint64_t kWorkspaceKept = 256ull << 20;
 std::mutex g_pool_mu;
 cudaMemPool_t g_pools[64] = {};
@@ -97,27 +108,15 @@ cudaMemPool_t workspace_pool() {
     }
     return g_pools[dev];
 }
+void workspace_trim() {
+    std::lock_guard<std::mutex> lock(g_pool_mu);
+    for (cudaMemPool_t p : g_pools)
+        if (p) cudaMemPoolTrimTo(p, 0);
+}
 sk_status ws_alloc(void** p, size_t bytes, cudaStream_t st) {
     const cudaError_t e = sk::workspace_alloc(p, bytes, st);
     if (e == cudaSuccess) return SK_OK;
     return fail(SK_ERR_OOM, "workspace of %zu bytes: %s", bytes, cudaGetErrorString(e));
-}
-
-template <typename T>
-sk_status dalloc(T** p, size_t bytes) {
-    *p = nullptr;
-    if (bytes == 0) return SK_OK;
-    cudaError_t e = cudaMalloc(reinterpret_cast<void**>(p), bytes);
-    if (e == cudaErrorMemoryAllocation) {  // what the workspace pool keeps is free memory too
-        cudaGetLastError();
-        sk::workspace_trim();
-        e = cudaMalloc(reinterpret_cast<void**>(p), bytes);
-    }
-    if (e != cudaSuccess) {
-        cudaGetLastError();
-        return fail(SK_ERR_OOM, "cudaMalloc(%zu) failed: %s", bytes, cudaGetErrorString(e));
-    }
-    return SK_OK;
 }
 
 // +-J weight tables (exact integer arithmetic on both the chain and its
@@ -203,11 +202,6 @@ std::vector<unsigned char> graph_table(uint32_t graph, uint32_t V, uint32_t arit
 
 namespace sk {
 void set_error_message(const char* msg) { g_err = msg; }
-void workspace_trim() {
-    std::lock_guard<std::mutex> lock(g_pool_mu);
-    for (cudaMemPool_t p : g_pools)
-        if (p) cudaMemPoolTrimTo(p, 0);
-}
 cudaError_t workspace_alloc(void** p, size_t bytes, cudaStream_t st) {
     *p = nullptr;
     cudaMemPool_t pool = workspace_pool();
@@ -735,7 +729,7 @@ sk_status sk_destroy_instance(sk_instance* in) {
     cudaEventDestroy(in->ev_main);
     cudaStreamDestroy(in->side);
     delete in;
-    if (--g_instances == 0) sk::workspace_trim();
+    if (--g_instances == 0) workspace_trim();
     return SK_OK;
 }
 

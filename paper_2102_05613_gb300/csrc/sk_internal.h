@@ -316,8 +316,6 @@ bool root_setup(JobDev& j, uint32_t K, double p_center);
 // Stream-ordered workspace from the library's pool of the current device
 // (sk_capi.cu); released with cudaFreeAsync.
 cudaError_t workspace_alloc(void** p, size_t bytes, cudaStream_t st);
-// Gives back what the pools keep and no call uses.
-void workspace_trim();
 
 // Sets the message sk_last_error() returns on this thread (sk_capi.cu).
 void set_error_message(const char* msg);

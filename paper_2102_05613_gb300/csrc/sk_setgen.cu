@@ -255,18 +255,6 @@ __global__ void setgen_ends(double* out, uint32_t all) {
     }
 }
 
-// cudaMalloc, once more after the workspace pool's kept memory has gone back.
-template <typename T>
-cudaError_t alloc(T** p, size_t bytes) {
-    cudaError_t e = cudaMalloc(p, bytes);
-    if (e == cudaErrorMemoryAllocation) {
-        cudaGetLastError();
-        workspace_trim();
-        e = cudaMalloc(p, bytes);
-    }
-    return e;
-}
-
 // The block form on the host side; out: 2^n doubles on the host or the device.
 cudaError_t setgen_blocks(uint32_t n, const double* P, double* out, bool host, cudaStream_t st) {
     const uint32_t L = n < kLow ? n : kLow, S = 1u << L, H = n - L;
@@ -291,7 +279,7 @@ cudaError_t setgen_blocks(uint32_t n, const double* P, double* out, bool host, c
     unsigned char* d = nullptr;
     double* dout = host ? nullptr : out;
     cudaError_t e = workspace_alloc(reinterpret_cast<void**>(&d), o_B + n * (static_cast<size_t>(S) + (1u << H1) + (1u << (H - H1))) * sizeof(double), st);
-    if (e == cudaSuccess && host) e = alloc(&dout, sizeof(double) << n);
+    if (e == cudaSuccess && host) e = cudaMalloc(&dout, sizeof(double) << n);
     if (e == cudaSuccess) e = cudaMemcpyAsync(d, up.data(), o_B, cudaMemcpyHostToDevice, st);
     if (e == cudaSuccess) {
         const double* dP = reinterpret_cast<const double*>(d);
@@ -358,16 +346,16 @@ extern "C" sk_status sk_set_generation(uint32_t n, const double* P, double* out,
     double* dout = mem == SK_MEM_DEVICE ? out : nullptr;
     cudaError_t e = cudaSuccess;
     if (method == SK_SETGEN_CUMULATIVE && n > 1) {
-        e = sk::alloc(&dc, nmask * n * sizeof(double));
+        e = cudaMalloc(&dc, nmask * n * sizeof(double));
         if (e != cudaSuccess) {
             cudaGetLastError();
             sk::set_error_message("sk_set_generation: no room for the cumulative table (n 2^n doubles)");
             return SK_ERR_OOM;
         }
     }
-    if (e == cudaSuccess) e = sk::alloc(&dP, n * n * sizeof(double));
-    if (e == cudaSuccess) e = sk::alloc(&dC, C.size() * sizeof(unsigned long long));
-    if (e == cudaSuccess && !dout) e = sk::alloc(&dout, nmask * sizeof(double));
+    if (e == cudaSuccess) e = cudaMalloc(&dP, n * n * sizeof(double));
+    if (e == cudaSuccess) e = cudaMalloc(&dC, C.size() * sizeof(unsigned long long));
+    if (e == cudaSuccess && !dout) e = cudaMalloc(&dout, nmask * sizeof(double));
     if (e == cudaSuccess) e = cudaMemcpyAsync(dP, P, n * n * sizeof(double), cudaMemcpyHostToDevice, st);
     if (e == cudaSuccess) e = cudaMemcpyAsync(dC, C.data(), C.size() * sizeof(unsigned long long), cudaMemcpyHostToDevice, st);
     if (e == cudaSuccess) {
