@@ -1397,15 +1397,22 @@ bool plan_team_class(const sk_batch* b, const std::vector<uint32_t>& idx, uint32
 // for a layout (0: the warp layouts).  Results are the same either way.  A
 // team shortens a chain's step, so it is taken where the batch's chains are so
 // few that all are in flight in one round of the class's CTAs.  ns a step, one
-// warp / 2 warps / 4 warps per chain, one chain and 304 chains, N = 512 (2048):
-//   Metropolis, Gaussian  287 / 190 / 189;  309 / 206 / 210 (356 / 285 / 230)
-//   K = 8, Gaussian       843 / 733 / 748;  886 / 792 / 788 (1259 / 988 / 860)
-//   K = 64                1221 / 943 / 919;  1278 / 1001 / 983 (1895 / 1353 / 1130)
-//   K = 128               1254 / - / 945;  1295 / - / 1010 (2016 / - / 1194)
-// and beyond: 608 chains K = 64 1283 / 1043 / 1949 (two rounds), 1216 chains
-// Metropolis 324 / 240 / 449.  +-J runs whose weight
-// table fits the shared copy have a one-warp loop of their own, the faster one
-// up to K = 32 (K = 8 512 / 685, K = 32 553 / 657; K = 64 819 / 705).
+// warp / 2 warps / 4 warps per chain, 600 steps from a random start with their
+// launch; one chain and 304 chains at N = 512, 304 at 2048:
+//   Metropolis, Gaussian  360 / 244 / 242;  398 / 264 / 268;  573 / 485 / 368
+//   K = 8, Gaussian       895 / 803 / 793;  962 / 859 / 856;  1709 / 1336 / 1129
+//   K = 64                1205 / 1036 / 999;  1226 / 1068 / 1045;  2073 / 1602 / 1352
+//   K = 128               1219 / - / 991;  1263 / - / 1067;  2124 / - / 1372
+// and beyond, N = 512: 600 chains K = 64 1228 / 1112 / 2061 (two rounds), 1000
+// chains Metropolis 420 / 300 / 544.  +-J runs whose weight table fits the
+// shared copy have one-warp loops of their own.  They are the faster ones for
+// K <= 32 at N = 512 (K = 8 728 / 801 / 793, K = 32 787 / 804 / 790) and for K of
+// 33 to 64 below N = 1024 (K = 64, one chain and 600: N = 128 639 / 735 / 718, 654 /
+// 804 / 1530; N = 512 835 / 869 / 834, 872 / 955 / 1750; N = 768 1088 / 1118 / 1044,
+// 1127 / 1232 / 2204), at N = 1024 still for what exceeds the 4-warp teams (304
+// chains 1272 / 1249 / 1199, 600 1274 / 1325 / 2345; N = 2048 1881 / 1591 / 1382, 1895 /
+// 1696 / 2721).  +-J Metropolis steps of N >= 1024 beyond the 4-warp teams: 600
+// chains N = 1024 346 / 355, N = 4096 886 / 910, a longer table 849 / 957.
 uint32_t default_team(const sk_batch* b, const std::vector<uint32_t>& idx, int sms) {
     const sk_run* r0 = b->runs[idx[0]];
     if (run_nw(r0) || r0->p.graph) return 0;
@@ -1421,12 +1428,14 @@ uint32_t default_team(const sk_batch* b, const std::vector<uint32_t>& idx, int s
         short_tables = short_tables && r->wlen <= 64u;
         single = single && r->chains == 1;
     }
-    if (K > 128u || (short_tables && r0->p.rule == SK_RULE_MCMCMC && K <= 32u)) return 0;
+    const bool metropolis = r0->p.rule == SK_RULE_METROPOLIS;
+    if (K > 128u || (short_tables && !metropolis && (K <= 32u || (K <= 64u && npad < 1024u)))) return 0;
     const uint32_t per_cta = single ? 1u : 2u;
     const uint64_t s = static_cast<uint64_t>(sms);
     // 4 warps: one CTA per SM; 2 warps: two (Metropolis, fewer registers: four)
     if (total <= per_cta * s && (K > 64u || npad >= 1024u)) return 4;
-    if (K <= 64u && total <= (r0->p.rule == SK_RULE_METROPOLIS ? 4u : 2u) * per_cta * s) return 2;
+    if (metropolis ? r0->inst->kind == SK_J_PM1 && npad >= 1024u : short_tables && npad < 2048u) return 0;
+    if (K <= 64u && total <= (metropolis ? 4u : 2u) * per_cta * s) return 2;
     return 0;
 }
 

@@ -125,3 +125,22 @@ inst.close()
 """
     r = subprocess.run([sys.executable, "-c", code], cwd=ROOT, capture_output=True, text=True, timeout=300)
     assert r.returncode == 0, r.stderr[-2000:]
+
+
+@pytest.mark.parametrize("N,chains,K,rule,lanes", [
+    (128, 1, 33, 0, 32), (512, 304, 64, 0, 32), (768, 600, 48, 0, 32), (1024, 304, 48, 0, 128), (1024, 600, 48, 0, 32),
+    (2048, 600, 64, 0, 64), (512, 1, 100, 0, 128), (512, 304, 1, 1, 64), (1024, 304, 1, 1, 128), (1024, 600, 1, 1, 32)])
+def test_default_of_few_pm1_chains(N, chains, K, rule, lanes):
+    # +-J chains whose weight table is short got teams where their one-warp
+    # loop is the faster one; either layout gives the oracle's chain
+    need_gpu()
+    J = inputs.couplings_pm1(N, 95)
+    init = inputs.initial_spins(chains, N, 96)
+    inst = sk.Instance(J)
+    run = sk.Run(inst, chains=chains, K=K, rule=rule, beta=1.0, seed=97, init=init)
+    b = sk.Batch([run])
+    assert b.classes()[0][1] == lanes, b.classes()
+    b.advance(30)
+    o = oracle.run(J, K=K, rule=rule, beta=1.0, seed=97, chains=chains, init=init, steps=30)
+    assert np.array_equal(run.state()[0], o["spins"])
+    b.close(); run.close(); inst.close()
