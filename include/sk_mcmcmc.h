@@ -141,8 +141,12 @@ sk_status sk_destroy_instance(sk_instance* inst);
 
 /*
  * sk_energy: E(s) = -scale sum_{i<j} J_ij s_i s_j for `count` configurations
- * (Sec. IV.A), computed on the device in double precision (exact for +-J).
- *   spins  count*N int8 values +-1, row-major (mem: SK_MEM_HOST/DEVICE);
+ * (Sec. IV.A), computed on the device: exact for +-J; Gaussian as exact integer
+ * sums rounded at the end, or in double precision where calls are small, there
+ * is no room for the operands or the couplings span more than 62 bits.
+ *   spins  count*N int8 values +-1, row-major (mem: SK_MEM_HOST/DEVICE); other
+ *          values are refused on the host, on the device one below 0 counts
+ *          as -1 and any other as +1;
  *   out_E  count doubles, always a host pointer.
  */
 sk_status sk_energy(const sk_instance* inst, const int8_t* spins, uint32_t count, uint32_t mem,
@@ -661,7 +665,9 @@ typedef struct {
  * first in first out, while their device footprint (couplings and their
  * tensor-core operand unless already resident, the run's memory as listed
  * under mcmcmc_create) fits
- * `budget_bytes`; each quantum advances every admitted job in one launch per
+ * `budget_bytes`; the workspace of a retiring job's energies (up to ~300 MB while
+ * they are computed) is not charged, but the library keeps no more of it
+ * than the budget leaves; each quantum advances every admitted job in one launch per
  * kernel class.  A job's result does not depend on the other jobs it shared
  * launches with (counter-based draws).  The paper's problem statement
  * (Sec. II) applied to many independent requests.

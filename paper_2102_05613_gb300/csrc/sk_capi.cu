@@ -83,8 +83,9 @@ sk_status dalloc(T** p, size_t bytes) {
 // between calls (a cudaMalloc / cudaFree pair of the 80 MB an energy call at
 // N = 2048 takes costs more than its kernels), more goes back at the next
 // synchronisation, and all of it when the process's last instance is
-// destroyed.  The runtime's pools are safe for concurrent threads and order
-// reuse between streams.
+// destroyed (set generation, which takes less than 1 MB, needs no instance and
+// can leave that).  The runtime's pools are safe for concurrent threads and
+// order reuse between streams.
 constexpr uint64_t kWorkspaceKept = 256ull << 20;
 std::mutex g_pool_mu;
 cudaMemPool_t g_pools[64] = {};
@@ -107,11 +108,6 @@ cudaMemPool_t workspace_pool() {
         }
     }
     return g_pools[dev];
-}
-void workspace_trim() {
-    std::lock_guard<std::mutex> lock(g_pool_mu);
-    for (cudaMemPool_t p : g_pools)
-        if (p) cudaMemPoolTrimTo(p, 0);
 }
 sk_status ws_alloc(void** p, size_t bytes, cudaStream_t st) {
     const cudaError_t e = sk::workspace_alloc(p, bytes, st);
@@ -202,6 +198,17 @@ std::vector<unsigned char> graph_table(uint32_t graph, uint32_t V, uint32_t arit
 
 namespace sk {
 void set_error_message(const char* msg) { g_err = msg; }
+uint64_t workspace_held() {
+    cudaMemPool_t pool = workspace_pool();
+    uint64_t n = 0;
+    if (pool && cudaMemPoolGetAttribute(pool, cudaMemPoolAttrReservedMemCurrent, &n) != cudaSuccess) cudaGetLastError();
+    return n;
+}
+void workspace_trim() {
+    std::lock_guard<std::mutex> lock(g_pool_mu);
+    for (cudaMemPool_t p : g_pools)
+        if (p) cudaMemPoolTrimTo(p, 0);
+}
 cudaError_t workspace_alloc(void** p, size_t bytes, cudaStream_t st) {
     *p = nullptr;
     cudaMemPool_t pool = workspace_pool();
@@ -729,7 +736,7 @@ sk_status sk_destroy_instance(sk_instance* in) {
     cudaEventDestroy(in->ev_main);
     cudaStreamDestroy(in->side);
     delete in;
-    if (--g_instances == 0) workspace_trim();
+    if (--g_instances == 0) sk::workspace_trim();
     return SK_OK;
 }
 

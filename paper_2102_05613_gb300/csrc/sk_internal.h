@@ -316,6 +316,10 @@ bool root_setup(JobDev& j, uint32_t K, double p_center);
 // Stream-ordered workspace from the library's pool of the current device
 // (sk_capi.cu); released with cudaFreeAsync.
 cudaError_t workspace_alloc(void** p, size_t bytes, cudaStream_t st);
+// Bytes the current device's pool holds, in use or kept between calls; giving
+// back what is not in use.
+uint64_t workspace_held();
+void workspace_trim();
 
 // Sets the message sk_last_error() returns on this thread (sk_capi.cu).
 void set_error_message(const char* msg);

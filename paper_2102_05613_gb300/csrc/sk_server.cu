@@ -115,9 +115,18 @@ bool fits(sk_server* s, const Job& j) {
     return s->used + need <= s->budget;
 }
 
+// The library's workspace pool (the operands of retiring jobs' energies) keeps
+// no more between calls than the budget leaves once `need` more bytes are used.
+// The workspace itself is not charged: which form the energies take must not
+// depend on the other jobs.
+void trim_to_budget(const sk_server* s, uint64_t need) {
+    if (s->used + need + sk::workspace_held() > s->budget) sk::workspace_trim();
+}
+
 sk_status admit(sk_server* s, Job& j) {
     sk_status r = SK_OK;
     sk_instance* inst = nullptr;
+    trim_to_budget(s, j.run_bytes + j.inst_bytes);
     if (j.spec.couplings_id) {
         Resident* res;
         {
@@ -207,6 +216,7 @@ void retire(sk_server* s, Job& j) {
     sk_status r = mcmcmc_state(j.run, j.spins.data(), nullptr, nullptr, SK_MEM_HOST);
     sk_instance* inst = j.own_inst ? j.own_inst : j.shared->inst;
     if (r == SK_OK) r = sk_energy(inst, j.spins.data(), static_cast<uint32_t>(C), SK_MEM_HOST, j.energies.data());
+    trim_to_budget(s, 0);
     if (r == SK_OK) r = mcmcmc_counters(j.run, &j.flips, nullptr);
     release(s, j);
     std::lock_guard<std::mutex> lk(s->mu);

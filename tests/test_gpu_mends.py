@@ -144,3 +144,30 @@ def test_default_of_few_pm1_chains(N, chains, K, rule, lanes):
     o = oracle.run(J, K=K, rule=rule, beta=1.0, seed=97, chains=chains, init=init, steps=30)
     assert np.array_equal(run.state()[0], o["spins"])
     b.close(); run.close(); inst.close()
+
+
+@pytest.mark.parametrize("spare", [2 << 20, 80 << 20])
+def test_server_keeps_no_workspace_beyond_its_budget(spare):
+    # the pool of the operands of retiring jobs' energies stayed with the process
+    # on top of budget_bytes
+    torch = need_gpu()
+    N, chains = 1024, 2048
+    job = dict(couplings_id=1, N=N, kind=sk.SK_J_GAUSS, chains=chains, steps=20, K=8, seed=4)
+
+    def go(budget):
+        torch.cuda.synchronize()
+        free = torch.cuda.mem_get_info()[0]
+        srv = sk.Server(budget_bytes=budget, quantum_steps=20)
+        srv.add_couplings(1, inputs.couplings(N, sk.SK_J_GAUSS, 98))
+        t = srv.submit(**job)
+        srv.wait_all()
+        held = free - torch.cuda.mem_get_info()[0]
+        footprint = srv.poll(t)["footprint_bytes"]
+        out = srv.result(t, chains, N)
+        srv.close()
+        return held, footprint, out
+
+    _, footprint, first = go(1 << 30)  # (loads the kernels)
+    held, _, out = go(footprint + spare)
+    assert held <= footprint + spare, (held, footprint, spare)
+    assert all(np.array_equal(x, y) for x, y in zip(out, first))
