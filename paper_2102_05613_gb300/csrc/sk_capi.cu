@@ -440,14 +440,27 @@ sk_status upload_couplings(sk_instance* in, const void* J, uint32_t mem, bool fr
     return couplings_commit(in, fresh);
 }
 
+// Waits for a stream: polls it without a pause for the first 20 ms (a sleep
+// of 50 us costs a short run as much as its launches), then every 50 us, so
+// that a run of minutes does not hold a host core.
+cudaError_t wait_stream(cudaStream_t st) {
+    const auto t0 = std::chrono::steady_clock::now();
+    bool spin = true;
+    for (;;) {
+        const cudaError_t e = cudaStreamQuery(st);
+        if (e != cudaErrorNotReady) return e;
+        if (spin) spin = std::chrono::steady_clock::now() - t0 < std::chrono::milliseconds(20);
+        if (!spin) std::this_thread::sleep_for(std::chrono::microseconds(50));
+    }
+}
+
 // Waits for the run's stream and reports an error its kernels left: the copy
 // of the error word (into pinned memory) is queued behind the work and one
-// wait covers both.  (Polling the stream with 50 us sleeps and then copying
-// the word into pageable memory cost a short run 50 to 100 us.)
+// wait covers both.
 sk_status check_run_error(sk_run* r) {
     int* herr = reinterpret_cast<int*>(r->hflag + 1);
     SK_CU(cudaMemcpyAsync(herr, r->derr, sizeof(int), cudaMemcpyDeviceToHost, r->inst->st));
-    SK_CU(cudaStreamSynchronize(r->inst->st));
+    SK_CU(wait_stream(r->inst->st));
     const int h = *herr;
     if (h == sk::kDevTimeout) return fail(SK_ERR_TIMEOUT, "a bounded device wait expired in the step kernel");
     if (h == sk::kDevBounds) return fail(SK_ERR_DEVICE, "a kernel reported an out-of-range index");

@@ -2,6 +2,7 @@
 import os
 import subprocess
 import sys
+import time
 
 import numpy as np
 import pytest
@@ -171,3 +172,19 @@ def test_server_keeps_no_workspace_beyond_its_budget(spare):
     held, _, out = go(footprint + spare)
     assert held <= footprint + spare, (held, footprint, spare)
     assert all(np.array_equal(x, y) for x, y in zip(out, first))
+
+
+def test_wait_without_a_limit_does_not_hold_a_core():
+    # the wait for a long run polled or synchronised without a pause
+    need_gpu()
+    inst = sk.Instance(inputs.couplings_pm1(64, 1))
+    run = sk.Run(inst, chains=1, K=8, beta=1.0, seed=2)
+    run.advance(100)
+    run.wait()
+    run.advance(1_000_000)
+    w0, c0 = time.perf_counter(), time.thread_time()
+    run.wait()
+    wall, cpu = time.perf_counter() - w0, time.thread_time() - c0
+    assert wall > 0.2 and cpu < 0.5 * wall, (wall, cpu)
+    assert run.state()[1] == 1_000_100
+    run.close(); inst.close()
