@@ -318,3 +318,52 @@ def test_reset_many_by_stream_and_kind():
         r.close()
     for x in insts:
         x.close()
+
+
+def test_reset_many_of_long_gaussian_runs():
+    # restarts of one stream together, sized for the 256-row tiles of the field
+    # launch (two rounds of 128-row tiles on 152 SMs, one of 256-row ones): uneven N,
+    # last tiles with 100 rows (none in the second half), with 130 and with 2
+    torch = need_gpu()
+    specs = [(1024, 2660), (1500, 1410), (1100, 130), (1030, 258)]
+    runs, insts, inits = [], [], []
+    for i, (N, chains) in enumerate(specs):
+        insts.append(sk.Instance(inputs.couplings(N, sk.SK_J_GAUSS, 800 + i)))
+        runs.append(sk.Run(insts[-1], chains=chains, K=8, seed=3, stream_id=i))
+        inits.append(inputs.initial_spins(chains, N, 810 + i))
+    for r in runs:
+        r.advance(3)
+    sk.reset_many(runs, inits)
+    for i, ((N, chains), r) in enumerate(zip(specs, runs)):
+        s, h, step = r.state(fields=True)
+        exact = torch.from_numpy(inits[i]).cuda().double() @ torch.from_numpy(inputs.couplings(N, sk.SK_J_GAUSS, 800 + i)).cuda().double()
+        err = (torch.from_numpy(h).cuda().double() - exact).abs().max().item()
+        # the tensor core's FP32 accumulator rounds once per MMA step of 16 products
+        assert step == 0 and np.array_equal(s, inits[i]) and err <= max(3e-5, 3 * N / 16 * 2.0 ** -23 * 4), (N, err)
+    for x in runs + insts:
+        x.close()
+
+
+@pytest.mark.parametrize("scale", [1.0, 0.1])
+@pytest.mark.parametrize("rule,K,N,chains,lanes", [
+    (0, 5, 33, 9001, 8), (0, 32, 250, 9001, 8), (0, 33, 130, 9001, 16), (0, 64, 256, 9001, 16), (0, 65, 77, 5017, 16),
+    (0, 128, 130, 20001, 16), (1, 1, 250, 9001, 16), (0, 48, 128, 20001, 32), (0, 20, 300, 5017, 32)])
+def test_default_layout_of_many_pm1_chains(rule, K, N, chains, lanes, scale):
+    # the lanes +-J chains get by default beyond 32 per SM (short and long weight
+    # tables), against the oracle; ragged N, K and last item
+    need_gpu()
+    steps = 24
+    J = inputs.couplings_pm1(N, 75)
+    init = inputs.initial_spins(chains, N, 76)
+    inst = sk.Instance(J, scale=scale)
+    run = sk.Run(inst, chains=chains, K=K, rule=rule, beta=1.2, seed=77, record_every=8, max_records=3, init=init)
+    b = sk.Batch([run])
+    assert b.classes()[0][1] == lanes, b.classes()
+    for n in (1, 16, 7):
+        b.advance(n)
+    E, q, acc = run.observables()
+    o = oracle.run(J, K=K, rule=rule, beta=1.2, seed=77, chains=chains, init=init, steps=steps, record_every=8,
+                   scale=scale)
+    assert np.array_equal(E, o["E"]) and np.array_equal(q, o["q"]) and np.array_equal(acc, o["acc"])
+    assert np.array_equal(run.state()[0], o["spins"])
+    b.close(); run.close(); inst.close()
