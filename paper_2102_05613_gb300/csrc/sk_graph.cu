@@ -520,8 +520,9 @@ __device__ __forceinline__ void graph_loop(const JobDev& jb, bool write, uint32_
         }
         team_sync(nw, team);
         // fields: h_k -= 2 sum_i fs_i J[fx_i][k], four elements per thread,
-        // the rows' loads issued eight flips at a time (a binary tree of depth 7 moves ~10:
-        // two round trips to L2 where four at a time took three)
+        // the rows' loads issued eight flips at a time for Gaussian J (a binary tree of depth 7
+        // moves ~10: two round trips to L2 where four at a time took three), the rest by up to 7 or
+        // 3 rows (a tree of 7 nodes, N = 1024, 3000 chains: 8.9 us a step, 10.0 with 7 only)
         for (uint32_t k = 4u * tid; k < npad; k += 4u * T) {
             const JT* col = Jg + k;
             if constexpr (sizeof(JT) == 1) {
@@ -532,25 +533,29 @@ __device__ __forceinline__ void graph_loop(const JobDev& jb, bool write, uint32_
                     hv.z -= c * dev::sbyte(j, 2);
                     hv.w -= c * dev::sbyte(j, 3);
                 };
+                // (four at a time: a lane's int8 rows are one word each, and
+                // with eight the rest's predicated rows cost small trees of
+                // many chains more, N = 1024, 7 nodes, 3000 chains 9.2 -> 10.7 us
+                // a step, 63 nodes 21.4 -> 24.6, than the longest moves gain)
                 uint32_t i = 0;
-                for (; i + 8u <= n; i += 8u) {
-                    uint32_t j[8];
+                for (; i + 4u <= n; i += 4u) {
+                    uint32_t j[4];
 #pragma unroll
-                    for (int q = 0; q < 8; ++q)
+                    for (int q = 0; q < 4; ++q)
                         j[q] = __ldg(reinterpret_cast<const unsigned int*>(col + static_cast<size_t>(lx[i + q]) * npad));
 #pragma unroll
-                    for (int q = 0; q < 8; ++q) upd(j[q], 2 * ls[i + q]);
+                    for (int q = 0; q < 4; ++q) upd(j[q], 2 * ls[i + q]);
                 }
-                if (i < n) {  // the last n - i < 8 rows together
+                if (i < n) {  // the last n - i < 4 rows together
                     const uint32_t r = n - i;
-                    uint32_t j[7];
+                    uint32_t j[3];
 #pragma unroll
-                    for (uint32_t q = 0; q < 7u; ++q)
+                    for (uint32_t q = 0; q < 3u; ++q)
                         j[q] = q < r ? __ldg(reinterpret_cast<const unsigned int*>(
                                            col + static_cast<size_t>(lx[i + q]) * npad))
                                      : 0u;
 #pragma unroll
-                    for (uint32_t q = 0; q < 7u; ++q)
+                    for (uint32_t q = 0; q < 3u; ++q)
                         if (q < r) upd(j[q], 2 * ls[i + q]);
                 }
                 *reinterpret_cast<int4*>(hf + k) = hv;
@@ -571,17 +576,20 @@ __device__ __forceinline__ void graph_loop(const JobDev& jb, bool write, uint32_
 #pragma unroll
                     for (int q = 0; q < 8; ++q) upd(j[q], static_cast<float>(2 * ls[i + q]));
                 }
-                if (i < n) {  // the last n - i < 8 rows together
+                auto rest = [&](auto most) {
+                    constexpr uint32_t M = decltype(most)::value;
                     const uint32_t r = n - i;
-                    float4 j[7];
+                    float4 j[M];
 #pragma unroll
-                    for (uint32_t q = 0; q < 7u; ++q)
+                    for (uint32_t q = 0; q < M; ++q)
                         j[q] = q < r ? __ldg(reinterpret_cast<const float4*>(col + static_cast<size_t>(lx[i + q]) * npad))
                                      : make_float4(0.f, 0.f, 0.f, 0.f);
 #pragma unroll
-                    for (uint32_t q = 0; q < 7u; ++q)
+                    for (uint32_t q = 0; q < M; ++q)
                         if (q < r) upd(j[q], static_cast<float>(2 * ls[i + q]));
-                }
+                };
+                if (n - i > 3u) rest(std::integral_constant<uint32_t, 7>{});
+                else if (i < n) rest(std::integral_constant<uint32_t, 3>{});
                 *reinterpret_cast<float4*>(hf + k) = hv;
             }
         }
