@@ -1599,15 +1599,20 @@ sk_status plan_batch(sk_batch* b) {
                 c.W = tg->second & 0xFFu;
             } else {
                 // Untuned: the warps per chain that finish the class first.  A
-                // launch takes ceil(chains / (SMs x chains per CTA)) rounds and
-                // a step of a round about 1/nw + 0.05 of the one-warp step (its
-                // node passes and field update spread over the team, its
-                // barriers do not): Gaussian N = 1024, binary depth 7, us a
-                // step at nw = 1, 2, 4, 8, 16: 152 chains 66, 32, 19, 11.8, 9.8;
-                // 4096 chains 137, 67, 76, 81, 130.  One warp counts for a
-                // quarter more: with a CTA full of one-warp chains the lanes
-                // of a warp wait for its longest path (the line of 128, 4096
-                // chains: 127 in one round against 71 in two of nw = 2).  No
+                // launch takes ceil(chains / (SMs x chains per CTA)) rounds; a
+                // step of a round takes a latency, of which the node passes
+                // and the field update spread over the chain's warps and the
+                // barriers do not, and issue time per warp in flight (every warp
+                // of a team scans, draws and waits for itself, so that more
+                // warps per chain issue more in all; a lone warp's lanes also
+                // wait for the longest of its paths).  The constants are fitted to 1830
+                // timings (trees of 7 to 585 nodes, lines of 8 to 128, N = 64 to
+                // 1024, both kinds, 1 to 12,000 chains, 1 to 16 warps; rms 14 %);
+                // the choice is within 22 % of the best form everywhere, 1 % on
+                // average.  us a step at 1, 2, 4, 8, 16 warps: Gaussian N = 1024,
+                // 255 nodes 152 chains 63, 31, 19, 12, 9.9, 6000 chains 145, 104,
+                // 104, 128, 208; +-J N = 300, 7 nodes, 3000 chains 7.0, 11.1, 16.5,
+                // 24.0, 50.6 (a rule without the issue term took 4 warps there).  No
                 // more warps than nodes or field words to give them.
                 uint64_t total = 0;
                 uint32_t most = 1;
@@ -1622,14 +1627,31 @@ sk_status plan_batch(sk_batch* b) {
                     return ch;
                 };
                 c.nw = b->G_override >= 64 ? std::min<uint32_t>(16, b->G_override / 32) : 1u;
+                // few chains: spread over the SMs, two per CTA at least
+                auto spread = [&](uint32_t ch) -> uint32_t {
+                    while (ch > 2 && total <= static_cast<uint64_t>(sms) * (ch - 2)) ch -= 2;
+                    return ch;
+                };
                 if (b->G_override == 0 && b->W_override == 0) {
+                    // q: J lookups of the nodes' paths; p: thousands of field
+                    // elements the move's rows change
+                    double q = 0.0, p = 0.0, far = 0.0;
+                    for (uint32_t i : g.second) {
+                        const sk_run* r = b->runs[i];
+                        const double V = r->job.V, N = r->inst->N;
+                        const bool tree = r->p.graph == SK_GRAPH_TREE;
+                        q = std::max(q, V * (tree ? r->p.depth : V / 12.0));
+                        p = std::max(p, 1e-3 * N * (tree ? 2.0 * r->p.depth : V / 3.0));
+                        far = std::max(far, std::min(1.0, N / 256.0));
+                    }
                     double best = 1e300;
                     for (uint32_t nw = 1; nw <= most; nw <<= 1) {
-                        const uint32_t ch = chains_of(nw);
-                        if (ch < 2) break;
+                        if (chains_of(nw) < 2) break;
+                        const uint32_t ch = spread(chains_of(nw));
                         const uint64_t per_round = static_cast<uint64_t>(sms) * ch;
-                        const double cost = static_cast<double>((total + per_round - 1) / per_round) *
-                                            (1.0 / nw + 0.05) * (nw == 1 ? 1.25 : 1.0);
+                        const double step = 3.6 + (0.0133 * q + 0.22 * p) / nw +
+                                            ch * nw * (0.034 + (4.8e-4 * q + 0.0154 * p) / nw + (nw == 1 ? 2.3e-4 * q * far : 0.0));
+                        const double cost = static_cast<double>((total + per_round - 1) / per_round) * step;
                         if (cost < best) {
                             best = cost;
                             c.nw = nw;
@@ -1638,9 +1660,7 @@ sk_status plan_batch(sk_batch* b) {
                 }
                 uint32_t chains = chains_of(c.nw);
                 if (chains < 2) return fail(SK_ERR_INVALID_ARG, "graph: %u warps per chain leave no room for two chains", c.nw);
-                // few chains: spread over the SMs, two per CTA at least
-                if (b->G_override == 0 && b->W_override == 0)
-                    while (chains > 2 && total <= static_cast<uint64_t>(sms) * (chains - 2)) chains -= 2;
+                if (b->G_override == 0 && b->W_override == 0) chains = spread(chains);
                 c.W = chains * c.nw;
             }
             if (!sk::graph_team_ok(c.W, c.nw)) return fail(SK_ERR_INVALID_ARG, "graph layout %u warps, %u per chain", c.W, c.nw);

@@ -188,3 +188,26 @@ def test_wait_without_a_limit_does_not_hold_a_core():
     assert wall > 0.2 and cpu < 0.5 * wall, (wall, cpu)
     assert run.state()[1] == 1_000_100
     run.close(); inst.close()
+
+
+@pytest.mark.parametrize("N,arity,depth,chains,nw", [(300, 2, 2, 3000, 1), (300, 2, 2, 12000, 1), (1024, 2, 3, 3000, 1),
+                                                     (1024, 2, 7, 32, 8), (1024, 2, 7, 6000, 2)])
+def test_default_warps_of_graph_chains(N, arity, depth, chains, nw):
+    # thousands of chains on small trees got 4 and 8 warps per chain, 1.6 to 2.9
+    # times the time of one; results are the oracle's either way
+    need_gpu()
+    J = inputs.couplings_pm1(N, 101)
+    init = inputs.initial_spins(chains, N, 102)
+    inst = sk.Instance(J)
+    run = sk.Run(inst, chains=chains, K=1, beta=0.05, seed=103, init=init, graph=sk.SK_GRAPH_TREE, arity=arity,
+                 depth=depth, trace_chains=chains, trace_steps=6)
+    b = sk.Batch([run])
+    got = b.classes()[0][1] // 32
+    assert got == 1 if nw == 1 else got >= nw, b.classes()
+    b.advance(6)
+    tr, s = run.trace(), run.state()[0]
+    n = min(chains, 40)
+    o = oracle.run_graph(J, graph=oracle.TREE, arity=arity, depth=depth, beta=0.05, seed=103, chains=n, init=init[:n],
+                         steps=6, trace=True)
+    assert np.array_equal(tr[:n], o["trace"]) and np.array_equal(s[:n], o["spins"])
+    b.close(); run.close(); inst.close()
