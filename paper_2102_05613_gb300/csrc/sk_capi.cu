@@ -1485,6 +1485,11 @@ uint32_t default_team(const sk_batch* b, const std::vector<uint32_t>& idx, int s
 // elsewhere.  A few rounds decide by the cost: CTA rounds times a round's
 // time, in whole-warp chains' worth of issue (12,288 Gaussian chains N = 512,
 // K = 128: three rounds of 28 warps 8.5 ms a 1000 steps, two of 16 lanes 7.6).
+// A Metropolis round of 16 lanes (64 chains per CTA) costs more of a whole-warp
+// round the longer the rows of its accepted steps are: from a random start,
+// 100 steps, 30,000 +-J chains at 32 / 16 lanes, N = 128 2.62 / 2.12 us a step,
+// 256 2.94 / 2.75, 400 4.21 / 4.39, 512 4.00 / 4.68 (1000 steps: 2.72 / 2.88);
+// Gaussian N = 256 3.53 / 3.55.
 struct ManyChains {
     uint32_t G = 0, W = 0;
 };
@@ -1510,7 +1515,7 @@ ManyChains many_chains_layout(const sk_batch* b, const std::vector<uint32_t>& id
     };
     // a round's fixed part, in chains: long Metropolis and short MCMCMC steps
     // wait more than they issue
-    const double fixed = metropolis ? 24.0 : K <= 32u ? 12.0 : 2.4;
+    const double fixed = metropolis ? 20.0 : K <= 32u ? 12.0 : 2.4;
     double cost = 1e300;
     const uint32_t fit32 = std::min(32u, fit_warps(per_chain, 32));
     if (fit32 < 18) return best;
@@ -1537,7 +1542,9 @@ ManyChains many_chains_layout(const sk_batch* b, const std::vector<uint32_t>& id
     const uint32_t spw = 32 / G;
     const uint32_t fit = std::min(most, fit_warps(per_chain, G));
     for (uint32_t W = fit; W > (!few ? fit - 1u : G == 8 ? 15u : 16u); --W) {
-        const double t = rounds(spw * W) * (G == 8 ? 66.0 : 0.42 * spw * W + (most > 24 ? 35.0 : 22.0));
+        const double t = rounds(spw * W) * (metropolis ? (0.55 + 0.00083 * npad + (pm1 ? 0.0 : 0.11)) * (spw * W + 40.0)
+                                            : G == 8   ? 66.0
+                                                       : 0.42 * spw * W + (most > 24 ? 35.0 : 22.0));
         if (t < cost) {
             cost = t;
             best = ManyChains{G, W};
