@@ -663,7 +663,7 @@ __device__ __forceinline__ void chain_loop(const JobDev& jb, bool write, uint32_
     // (one chain, ns a step: Gaussian N = 512, K = 128 1251 -> 1172, K = 256
     // 1552 -> 1435; the uneven fused batch 3 %): not in the throughput
     // variants, nor in the +-J loop of one slot per lane (533 -> 549 at K = 8)
-    constexpr bool LEAN = KEEPW && !(SPL1 && sizeof(JT) == 1);
+    constexpr bool LEAN = KEEPW && RULE == 0 && !(SPL1 && sizeof(JT) == 1);
     constexpr int NQ = SPL1 ? 1 : SPL2 ? 2 : 4 * NB;  // slots per lane
     constexpr int SCANL = SPL1 ? (4 * SL < G ? 4 * SL : G) : (SL > 0 ? SL : 1);
     const Grp<G> g;
