@@ -809,9 +809,9 @@ sk_status sk_energy(const sk_instance* in, const int8_t* spins, uint32_t count, 
                               tiles > 1 ? reinterpret_cast<double*>(base + o_part) : nullptr, slices);
     if (e == cudaSuccess) e = cudaMemcpyAsync(hE.get(), dE, count * sizeof(double), cudaMemcpyDeviceToHost, in->st);
     if (e == cudaSuccess && err) e = cudaMemcpyAsync(&herr, err, sizeof herr, cudaMemcpyDeviceToHost, in->st);
-    cudaFreeAsync(ws, in->st);
     const cudaError_t e2 = cudaStreamSynchronize(in->st);
     if (e == cudaSuccess) e = e2;
+    cudaFreeAsync(ws, in->st);  // (nothing left to wait for)
     if (e != cudaSuccess) return fail(SK_ERR_CUDA, "sk_energy: %s", cudaGetErrorString(e));
     if (hflag != ~0ull) return fail(SK_ERR_INVALID_ARG, "spin %llu is not +-1", hflag >> 2);
     if (herr) return fail(SK_ERR_TIMEOUT, "sk_energy: a bounded device wait expired");

@@ -1004,9 +1004,11 @@ cudaError_t launch_recompute(uint32_t kind, const int8_t* s, void* h, float* out
 // them; q is written as signed base-256 digits, each exact in bf16, and a
 // digit's sums stay below 2^20 (128 x 8192), exact in the FP32 accumulator.
 // The digits' energy sums are integers (int32 per tile row, int64 per
-// configuration) joined in 128 bits, so the result is rounded once, where the
-// double-precision sum it replaces (energy_kernel) rounds at every term: the
-// error against a 64-bit product is the same 1.1e-16 (N = 2048).  Couplings
+// configuration) joined in 128 bits, so the sum is rounded once (twice from
+// 2^64 units of the lowest bit on) and once more by the scale, where the
+// double-precision sum it replaces (energy_kernel) rounds at every term: rms
+// relative error against 113-bit sums 7.5e-17 and 5.2e-17 (N = 1024, 2048), that
+// sum's 8.0e-17 and 1.0e-16.  Couplings
 // that span more than kEnergyBits bits take energy_kernel.  Bound: FP64 adds
 // run at 2 per clock and SM on this part; the 7 slices a Gaussian matrix of
 // N = 2048 needs are 3e10 bf16 multiply-adds for 2048 configurations (half

@@ -216,9 +216,9 @@ void retire(sk_server* s, Job& j) {
     sk_status r = mcmcmc_state(j.run, j.spins.data(), nullptr, nullptr, SK_MEM_HOST);
     sk_instance* inst = j.own_inst ? j.own_inst : j.shared->inst;
     if (r == SK_OK) r = sk_energy(inst, j.spins.data(), static_cast<uint32_t>(C), SK_MEM_HOST, j.energies.data());
-    trim_to_budget(s, 0);
     if (r == SK_OK) r = mcmcmc_counters(j.run, &j.flips, nullptr);
     release(s, j);
+    trim_to_budget(s, 0);
     std::lock_guard<std::mutex> lk(s->mu);
     j.status.state = r == SK_OK ? SK_JOB_DONE : SK_JOB_FAILED;
     j.status.error = r;
