@@ -263,6 +263,9 @@ void loop(sk_server* s) {
             std::lock_guard<std::mutex> lk(s->mu);
             s->active.swap(still);
             s->retire_s += std::chrono::duration<double>(Clock::now() - tr0).count();
+            // a waiter that a retirement woke before this point found the job
+            // still in `active` and went back to waiting
+            if (s->active.empty()) s->done_cv.notify_all();
         }
         // 2. admit queued jobs that fit, first in first out
         {

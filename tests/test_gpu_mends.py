@@ -2,6 +2,7 @@
 import os
 import subprocess
 import sys
+import threading
 import time
 
 import numpy as np
@@ -211,3 +212,25 @@ def test_default_warps_of_graph_chains(N, arity, depth, chains, nw):
                          steps=6, trace=True)
     assert np.array_equal(tr[:n], o["trace"]) and np.array_equal(s[:n], o["spins"])
     b.close(); run.close(); inst.close()
+
+
+def test_wait_all_wakes_up():
+    # a waiter that took the lock between the last job's retirement and its
+    # leaving the active list waited for ever; several waiters, many bursts
+    need_gpu()
+    srv = sk.Server(budget_bytes=1 << 30, quantum_steps=8)
+    srv.add_couplings(1, inputs.couplings_pm1(64, 1))
+    for burst in range(250):
+        t = [srv.submit(couplings_id=1, N=64, kind=sk.SK_J_PM1, chains=2, steps=8, K=4, seed=1, stream_id=k)
+             for k in range(2)]
+        # (the condition holds when the limit is reached, so that a lost wake-up shows as a late return)
+        ws = [threading.Thread(target=srv.wait_all, args=(4_000_000_000,)) for _ in range(8)]
+        t0 = time.perf_counter()
+        for w in ws:
+            w.start()
+        for w in ws:
+            w.join()
+        assert time.perf_counter() - t0 < 3.0, burst
+        for x in t:
+            srv.result(x, 2, 64)
+    srv.close()
