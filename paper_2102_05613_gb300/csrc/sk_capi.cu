@@ -260,6 +260,7 @@ struct sk_batch {
         uint32_t per_chain;      // shared memory per chain
         uint32_t W;              // warps per CTA (cluster classes: chains per cluster)
         uint32_t nw = 1;         // graph classes: warps per chain
+        uint32_t V = 0;          // ... and nodes (the same for every run of a class)
         uint32_t first_item, n_items, grid;
         // cluster-per-chain layout: CTAs per cluster (0: a warp layout), the
         // J columns each CTA holds, the coupling kind, rule and Philox blocks
@@ -1592,6 +1593,7 @@ sk_status plan_batch(sk_batch* b) {
         }
         if ((c.key >> 59) & 1u) {  // graph runs: a team of nw warps per chain, an even number of chains per CTA
             c.graph = r0->p.graph;
+            c.V = r0->job.V;
             c.gmin = 32;
             c.stage = 0;
             c.per_chain = 0;
@@ -1673,10 +1675,10 @@ sk_status plan_batch(sk_batch* b) {
             if (!sk::graph_team_ok(c.W, c.nw)) return fail(SK_ERR_INVALID_ARG, "graph layout %u warps, %u per chain", c.W, c.nw);
             c.G = 32 * c.nw;
             c.cls = 512 + static_cast<int>(r0->inst->kind) * 4 + static_cast<int>(c.graph);
-            int occg = sk::graph_kernel_occupancy(r0->inst->kind, c.graph, c.W, c.nw, c.per_chain);
+            int occg = sk::graph_kernel_occupancy(r0->inst->kind, c.graph, r0->job.V, c.W, c.nw, c.per_chain);
             while (occg <= 0 && tg == b->tuned.end() && c.W > 2 * c.nw) {
                 c.W -= 2 * c.nw;
-                occg = sk::graph_kernel_occupancy(r0->inst->kind, c.graph, c.W, c.nw, c.per_chain);
+                occg = sk::graph_kernel_occupancy(r0->inst->kind, c.graph, r0->job.V, c.W, c.nw, c.per_chain);
             }
             if (occg <= 0) return fail(SK_ERR_CUDA, "graph kernel cannot be resident with %u warps", c.W);
             c.first_item = static_cast<uint32_t>(items.size());
@@ -2050,7 +2052,7 @@ sk_status launch_segment(sk_batch* b, uint64_t steps, int only = -1) {
                                         c.rule, c.team, c.W, c.per_chain, c.grid,
                                         static_cast<uint32_t>(b->runs.size()), last, cs)
             : c.graph ? sk::launch_graph(b->djobs, b->ditems + c.first_item, c.n_items, b->dqueue + k, steps, c.W,
-                                       c.nw, c.per_chain, c.grid, static_cast<uint32_t>((c.cls - 512) / 4), c.graph,
+                                       c.nw, c.per_chain, c.grid, static_cast<uint32_t>((c.cls - 512) / 4), c.graph, c.V,
                                        static_cast<uint32_t>(b->runs.size()), last, cs)
                     : sk::launch_step(b->djobs, b->ditems + c.first_item, c.n_items, b->dqueue + k, steps, c.W,
                                       c.per_chain, c.grid, c.cls, static_cast<uint32_t>(b->runs.size()), last, cs);

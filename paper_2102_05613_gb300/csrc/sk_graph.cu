@@ -176,8 +176,14 @@ __device__ __forceinline__ H path_dot(const JT* __restrict__ row, uint32_t n, co
     return acc;
 }
 
+// Whether the weights of a tree of V nodes are scanned in turned order (see graph_loop).
+bool turned_scan(uint32_t V) {
+    const uint32_t chunk = (V + 31u) / 32u;
+    return chunk >= 32u && !(chunk & 1u) && 32u * chunk <= ((V + 15u) & ~15u);
+}
+
 // One chain's steps t0..t1-1 by its team (T = 32 nw threads, tid in [0, T)).
-template <typename JT, int GRAPH>
+template <typename JT, int GRAPH, bool TURN>
 __device__ __forceinline__ void graph_loop(const JobDev& jb, bool write, uint32_t chain, const GMem& gm,
                                            int partner_off, uint32_t t0, uint32_t t1, uint32_t nw, uint32_t team,
                                            uint32_t& acc, uint32_t& n_flips) {
@@ -411,35 +417,94 @@ __device__ __forceinline__ void graph_loop(const JobDev& jb, bool write, uint32_
             // move.  (Before, each thread summed its own chunk and the warps'
             // totals met at two more barriers.)
             float* wv = reinterpret_cast<float*>(dl);
-            for (uint32_t v = tid; v < V; v += T) wv[v] = node_w(v);
-            team_sync(nw, team);
-            const uint32_t chunk = (V + 31u) / 32u, v0 = lane * chunk, v1 = min(V, v0 + chunk);
-            W lsum = W(0);
-            for (uint32_t v = v0; v < v1; ++v) lsum += wv[v];
-            const W incl = step::gscan(g, lsum);
-            const W total = __shfl_sync(kFull, incl, 31);
-            W u = static_cast<float>(U1 >> 40) * 0x1p-24f * total;
-            if (u >= total) u = nextafterf(total, 0.0f);
-            if (total > W(0) && u < total) {
-                const unsigned ball = __ballot_sync(kFull, incl > u);
-                const int L = ball ? __ffs(ball) - 1 : 31;
-                int found = -1, last = -1;
-                if (static_cast<int>(lane) == L) {
-                    // its first node whose prefix exceeds u (else, a rounding
-                    // guard, its last positive weight)
-                    W run = incl - lsum;
-                    for (uint32_t v = v0; v < v1; ++v) {
-                        const W x = wv[v];
-                        if (x > W(0)) {
-                            last = static_cast<int>(v);
-                            if (found < 0) {
-                                run += x;
-                                if (run > u) found = static_cast<int>(v);
+            const uint32_t chunk = (V + 31u) / 32u;
+            if constexpr (TURN) {
+                // an even chunk of many words puts the lanes on few banks (2047
+                // nodes: 64 words apart, all on one): each lane's words are turned
+                // round by its number, and read eight at a time.  Same sums.  N =
+                // 1024, 16 warps, 152 chains: 2047 nodes 84 -> 55 us a step, 4095 174
+                // -> 116.  (A kernel of its own, turned_scan: as a branch it cost small
+                // trees 3 to 7 %; eight words at a time for odd chunks gained nothing.)
+                const uint32_t kinv = 0xFFFFFFFFu / chunk + 1u;
+                auto turn = [&](uint32_t j, uint32_t l) -> uint32_t {
+                    const uint32_t p = j + l;
+                    return p >= chunk ? p - chunk : p;
+                };
+                for (uint32_t v = tid; v < V; v += T) {
+                    const uint32_t l = __umulhi(v, kinv);
+                    wv[l * chunk + turn(v - l * chunk, l)] = node_w(v);
+                }
+                team_sync(nw, team);
+                const float* wl = wv + lane * chunk;
+                const uint32_t v0 = lane * chunk, len = v0 < V ? min(V - v0, chunk) : 0u;
+                W lsum = W(0);
+                uint32_t j0 = 0;
+                for (; j0 + 8u <= len; j0 += 8u) {
+                    W x[8];
+#pragma unroll
+                    for (uint32_t e = 0; e < 8u; ++e) x[e] = wl[turn(j0 + e, lane)];
+#pragma unroll
+                    for (uint32_t e = 0; e < 8u; ++e) lsum += x[e];
+                }
+                for (; j0 < len; ++j0) lsum += wl[turn(j0, lane)];
+                const W incl = step::gscan(g, lsum);
+                const W total = __shfl_sync(kFull, incl, 31);
+                W u = static_cast<float>(U1 >> 40) * 0x1p-24f * total;
+                if (u >= total) u = nextafterf(total, 0.0f);
+                if (total > W(0) && u < total) {
+                    const unsigned ball = __ballot_sync(kFull, incl > u);
+                    const int L = ball ? __ffs(ball) - 1 : 31;
+                    int found = -1, last = -1;
+                    if (static_cast<int>(lane) == L) {
+                        // its first node whose prefix exceeds u (else, a rounding
+                        // guard, its last positive weight)
+                        W run = incl - lsum;
+                        for (uint32_t j = 0; j < len && found < 0; j += 8u) {
+                            W x[8];
+#pragma unroll
+                            for (uint32_t e = 0; e < 8u; ++e) x[e] = j + e < len ? wl[turn(j + e, lane)] : W(0);
+#pragma unroll
+                            for (uint32_t e = 0; e < 8u; ++e)
+                                if (x[e] > W(0)) {
+                                    last = static_cast<int>(v0 + j + e);
+                                    run += x[e];
+                                    if (found < 0 && run > u) found = static_cast<int>(v0 + j + e);
+                                }
+                        }
+                    }
+                    jsel = static_cast<uint32_t>(__shfl_sync(kFull, found >= 0 ? found : last, L));
+                }
+            } else {
+                for (uint32_t v = tid; v < V; v += T) wv[v] = node_w(v);
+                team_sync(nw, team);
+                const uint32_t v0 = lane * chunk, v1 = min(V, v0 + chunk);
+                W lsum = W(0);
+                for (uint32_t v = v0; v < v1; ++v) lsum += wv[v];
+                const W incl = step::gscan(g, lsum);
+                const W total = __shfl_sync(kFull, incl, 31);
+                W u = static_cast<float>(U1 >> 40) * 0x1p-24f * total;
+                if (u >= total) u = nextafterf(total, 0.0f);
+                if (total > W(0) && u < total) {
+                    const unsigned ball = __ballot_sync(kFull, incl > u);
+                    const int L = ball ? __ffs(ball) - 1 : 31;
+                    int found = -1, last = -1;
+                    if (static_cast<int>(lane) == L) {
+                        // its first node whose prefix exceeds u (else, a rounding
+                        // guard, its last positive weight)
+                        W run = incl - lsum;
+                        for (uint32_t v = v0; v < v1; ++v) {
+                            const W x = wv[v];
+                            if (x > W(0)) {
+                                last = static_cast<int>(v);
+                                if (found < 0) {
+                                    run += x;
+                                    if (run > u) found = static_cast<int>(v);
+                                }
                             }
                         }
                     }
+                    jsel = static_cast<uint32_t>(__shfl_sync(kFull, found >= 0 ? found : last, L));
                 }
-                jsel = static_cast<uint32_t>(__shfl_sync(kFull, found >= 0 ? found : last, L));
             }
             if (jsel >= V) jsel = root;  // no positive weight found (cannot happen for finite fields): stay
             if constexpr (GRAPH == 1) jdep = gm.fx[jsel];
@@ -624,7 +689,7 @@ __device__ __forceinline__ void graph_loop(const JobDev& jb, bool write, uint32_
     }
 }
 
-template <typename JT, int GRAPH, int MAXT>
+template <typename JT, int GRAPH, int MAXT, bool TURN>
 __global__ void __launch_bounds__(MAXT, 1)
     graph_kernel(const JobDev* __restrict__ jobs, const WorkItem* __restrict__ items, uint32_t n_items,
                  uint32_t* __restrict__ queue, uint32_t nsteps, uint32_t per_chain, uint32_t nw) {
@@ -665,7 +730,7 @@ __global__ void __launch_bounds__(MAXT, 1)
         __syncthreads();
         if (t1 > t0) {
             if (own) {
-                graph_loop<JT, GRAPH>(jb, true, chain, gm, partner_off, t0, t1, nw, team, acc, n_flips);
+                graph_loop<JT, GRAPH, TURN>(jb, true, chain, gm, partner_off, t0, t1, nw, team, acc, n_flips);
             } else {  // no chain in this team: meet the CTA's record barriers only
                 const uint32_t R = jb.record_every;
                 if (R)
@@ -692,24 +757,24 @@ __global__ void __launch_bounds__(MAXT, 1)
     }
 }
 
-template <typename JT, int GRAPH, int MAXT>
+template <typename JT, int GRAPH, int MAXT, bool TURN>
 cudaError_t launch_t(const JobDev* jobs, const WorkItem* items, uint32_t n_items, uint32_t* queue, uint32_t ns,
                      uint32_t W, uint32_t nw, uint32_t per_chain, uint32_t grid, cudaStream_t st) {
     const size_t smem = static_cast<size_t>(per_chain) * (W / nw);
-    cudaError_t e = cudaFuncSetAttribute(graph_kernel<JT, GRAPH, MAXT>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+    cudaError_t e = cudaFuncSetAttribute(graph_kernel<JT, GRAPH, MAXT, TURN>, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                          static_cast<int>(smem));
     if (e != cudaSuccess) return e;
-    graph_kernel<JT, GRAPH, MAXT><<<grid, 32 * W, smem, st>>>(jobs, items, n_items, queue, ns, per_chain, nw);
+    graph_kernel<JT, GRAPH, MAXT, TURN><<<grid, 32 * W, smem, st>>>(jobs, items, n_items, queue, ns, per_chain, nw);
     return cudaGetLastError();
 }
-template <typename JT, int GRAPH, int MAXT>
+template <typename JT, int GRAPH, int MAXT, bool TURN>
 int occupancy_t(uint32_t W, uint32_t nw, uint32_t per_chain) {
     const size_t smem = static_cast<size_t>(per_chain) * (W / nw);
     int n = 0;
-    if (cudaFuncSetAttribute(graph_kernel<JT, GRAPH, MAXT>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+    if (cudaFuncSetAttribute(graph_kernel<JT, GRAPH, MAXT, TURN>, cudaFuncAttributeMaxDynamicSharedMemorySize,
                              static_cast<int>(smem)) != cudaSuccess)
         return 0;
-    if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&n, graph_kernel<JT, GRAPH, MAXT>, 32 * W, smem) != cudaSuccess)
+    if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&n, graph_kernel<JT, GRAPH, MAXT, TURN>, 32 * W, smem) != cudaSuccess)
         return 0;
     return n;
 }
@@ -743,21 +808,21 @@ __global__ void bump_graph_steps(const JobDev* __restrict__ jobs, uint32_t n_job
 }  // namespace
 
 namespace {
-template <typename JT, int GRAPH>
+template <typename JT, int GRAPH, bool TURN = false>
 cudaError_t launch_g(const JobDev* jobs, const WorkItem* items, uint32_t n_items, uint32_t* queue, uint32_t ns,
                      uint32_t W, uint32_t nw, uint32_t per_chain, uint32_t grid, cudaStream_t st) {
-    return W <= 16 ? graphk::launch_t<JT, GRAPH, 512>(jobs, items, n_items, queue, ns, W, nw, per_chain, grid, st)
-                   : graphk::launch_t<JT, GRAPH, 1024>(jobs, items, n_items, queue, ns, W, nw, per_chain, grid, st);
+    return W <= 16 ? graphk::launch_t<JT, GRAPH, 512, TURN>(jobs, items, n_items, queue, ns, W, nw, per_chain, grid, st)
+                   : graphk::launch_t<JT, GRAPH, 1024, TURN>(jobs, items, n_items, queue, ns, W, nw, per_chain, grid, st);
 }
-template <typename JT, int GRAPH>
+template <typename JT, int GRAPH, bool TURN = false>
 int occupancy_g(uint32_t W, uint32_t nw, uint32_t pc) {
-    return W <= 16 ? graphk::occupancy_t<JT, GRAPH, 512>(W, nw, pc) : graphk::occupancy_t<JT, GRAPH, 1024>(W, nw, pc);
+    return W <= 16 ? graphk::occupancy_t<JT, GRAPH, 512, TURN>(W, nw, pc) : graphk::occupancy_t<JT, GRAPH, 1024, TURN>(W, nw, pc);
 }
 }  // namespace
 
 cudaError_t launch_graph(const JobDev* jobs, const WorkItem* items, uint32_t n_items, uint32_t* queue,
                          uint64_t nsteps, uint32_t W, uint32_t nw, uint32_t per_chain, uint32_t grid, uint32_t kind,
-                         uint32_t graph, uint32_t n_jobs, bool bump, cudaStream_t st) {
+                         uint32_t graph, uint32_t V, uint32_t n_jobs, bool bump, cudaStream_t st) {
     if (!graph_team_ok(W, nw) || (graph != 1u && graph != 2u)) return cudaErrorInvalidValue;
     cudaError_t e = cudaMemsetAsync(queue, 0, sizeof(uint32_t), st);
     if (e != cudaSuccess) return e;
@@ -765,6 +830,8 @@ cudaError_t launch_graph(const JobDev* jobs, const WorkItem* items, uint32_t n_i
     if (kind == 0)
         e = graph == 1u ? launch_g<int8_t, 1>(jobs, items, n_items, queue, ns, W, nw, per_chain, grid, st)
                         : launch_g<int8_t, 2>(jobs, items, n_items, queue, ns, W, nw, per_chain, grid, st);
+    else if (graph == 1u && graphk::turned_scan(V))
+        e = launch_g<float, 1, true>(jobs, items, n_items, queue, ns, W, nw, per_chain, grid, st);
     else
         e = graph == 1u ? launch_g<float, 1>(jobs, items, n_items, queue, ns, W, nw, per_chain, grid, st)
                         : launch_g<float, 2>(jobs, items, n_items, queue, ns, W, nw, per_chain, grid, st);
@@ -773,10 +840,11 @@ cudaError_t launch_graph(const JobDev* jobs, const WorkItem* items, uint32_t n_i
     return cudaGetLastError();
 }
 
-int graph_kernel_occupancy(uint32_t kind, uint32_t graph, uint32_t W, uint32_t nw, size_t per_chain) {
+int graph_kernel_occupancy(uint32_t kind, uint32_t graph, uint32_t V, uint32_t W, uint32_t nw, size_t per_chain) {
     if (!graph_team_ok(W, nw) || (graph != 1u && graph != 2u)) return 0;
     const uint32_t pc = static_cast<uint32_t>(per_chain);
     if (kind == 0) return graph == 1u ? occupancy_g<int8_t, 1>(W, nw, pc) : occupancy_g<int8_t, 2>(W, nw, pc);
+    if (graph == 1u && graphk::turned_scan(V)) return occupancy_g<float, 1, true>(W, nw, pc);
     return graph == 1u ? occupancy_g<float, 1>(W, nw, pc) : occupancy_g<float, 2>(W, nw, pc);
 }
 

@@ -249,8 +249,8 @@ size_t graph_table_bytes(uint32_t V);
 bool graph_team_ok(uint32_t W, uint32_t nw);
 cudaError_t launch_graph(const JobDev* jobs, const WorkItem* items, uint32_t n_items, uint32_t* queue,
                          uint64_t nsteps, uint32_t W, uint32_t nw, uint32_t per_chain, uint32_t grid, uint32_t kind,
-                         uint32_t graph, uint32_t n_jobs, bool bump, cudaStream_t st);
-int graph_kernel_occupancy(uint32_t kind, uint32_t graph, uint32_t W, uint32_t nw, size_t per_chain);
+                         uint32_t graph, uint32_t V, uint32_t n_jobs, bool bump, cudaStream_t st);
+int graph_kernel_occupancy(uint32_t kind, uint32_t graph, uint32_t V, uint32_t W, uint32_t nw, size_t per_chain);
 
 // Tensor-core field recompute (sk_recompute.cu).  Operand buffers: J as
 // e4m3 (+-J, npad^2 bytes) or three bf16 terms (Gaussian, 3 npad^2 x 2

@@ -234,3 +234,30 @@ def test_wait_all_wakes_up():
         for x in t:
             srv.result(x, 2, 64)
     srv.close()
+
+
+@pytest.mark.parametrize("arity,depth,lanes", [(2, 10, 512), (2, 10, 64), (2, 11, 0), (2, 9, 256), (3, 6, 512)])
+def test_graph_scan_of_large_trees(arity, depth, lanes):
+    # trees of 1024 nodes and more whose words per lane are even scan them in turned
+    # order (all lanes on one bank before: 1.5 times the step): same results as
+    # on one warp per chain, and the oracle's decisions
+    need_gpu()
+    N, chains, steps = 96, 3, 12
+    J = inputs.couplings_gauss(N, 111)
+    init = inputs.initial_spins(chains, N, 112)
+    outs = []
+    for lay in (32, lanes):
+        inst = sk.Instance(J)
+        run = sk.Run(inst, chains=chains, K=1, beta=0.8, seed=113, init=init, graph=sk.SK_GRAPH_TREE, arity=arity,
+                     depth=depth, trace_chains=chains, trace_steps=steps)
+        b = sk.Batch([run])
+        if lay:
+            b.set_layout(lanes=lay)
+        b.advance(steps)
+        outs.append((run.trace(),) + run.state(fields=True))
+        b.close(); run.close(); inst.close()
+    assert all(np.array_equal(x, y) for x, y in zip(*outs))
+    for c in range(chains):
+        r = oracle.replay_graph(J, outs[1][0][c], graph=oracle.TREE, arity=arity, depth=depth, line_nodes=2, beta=0.8,
+                                seed=113, chain=c, init=init[c], tol=1e-4)
+        assert r["bad"] == 0, (c, r)
